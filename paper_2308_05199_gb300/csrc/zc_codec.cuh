@@ -30,11 +30,10 @@
 
 #include <type_traits>
 
-#include "zc_device.cuh"
+#include "zc_rows.cuh"
 
 namespace zc {
 
-constexpr int GR = 8;                  // rows held in registers at a time
 constexpr int WSCAN = NTHREADS;        // warp units per width-scan chunk
 constexpr int DEC_U = 64;              // rows per warp unit of the decompressor
 // Batched decompression: items of at most this many decode tiles get no
@@ -112,7 +111,7 @@ struct Smem {
 __host__ __device__ constexpr int enc_slots(int U) { return U >= 128 ? 2 : 3; }
 constexpr int ENC_SLOTS_MAX = 3;
 constexpr int ENC_THREADS = NTHREADS + 32;
-constexpr int ENC_CTAS_PER_SM = 4;            // resident encoder CTAs per SM (registers)
+constexpr int ENC_CTAS_PER_SM = 3;            // resident encoder CTAs per SM (registers)
 constexpr unsigned BAR_ENCW = 1;              // named barrier: the encoder warps
 constexpr unsigned BAR_ENC = 2;               // + slot: tile encoded (resolver waits)
 constexpr unsigned BAR_RES = BAR_ENC + ENC_SLOTS_MAX;  // + slot: tile resolved (encoders wait)
@@ -121,37 +120,13 @@ __host__ __device__ constexpr unsigned long long ring_cta_bytes(int U)
 {
     return (unsigned long long)enc_slots(U) * NWARPS * seg_bytes(U);
 }
-// Rows of a warp unit staged in shared memory before a copy to the ring: the
-// whole unit up to 64 rows for the single-stream kernels (compress, scatter
-// pack), 32 rows at a time otherwise (16-chunk tiles, the batch kernel with
-// its many code paths, the fused ring step whose decoder metadata also takes
-// shared memory), so that 4 CTAs fit an SM; the stage holds their worst case
-// plus the carried partial 16 bytes.
-__host__ __device__ constexpr int stage_rows(int U, bool single) { return (single && U <= 64) ? U : 32; }
-__host__ __device__ constexpr int stage_bytes(int rows) { return seg_bytes(rows) + 16; }
-// Dynamic shared memory of an encoder CTA: width bytes of every slot and
-// warp, then every encoder warp's stage.
+// Dynamic shared memory of an encoder CTA: every encoder warp's two group
+// buffers, then the width bytes of every slot and warp.
 __host__ __device__ constexpr int enc_wb_bytes(int U) { return enc_slots(U) * NWARPS * U * 2; }
-// (The single-stream kernels take their stages in dynamic shared memory;
-// the others in a static array of 32-row stages, which leaves the driver
-// free to give the rest of the SM's memory to L1.)
-__host__ __device__ constexpr int enc_smem_bytes(int U, bool single = false)
-{
-    return enc_wb_bytes(U) + (single ? NWARPS * stage_bytes(stage_rows(U, true)) : 0);
-}
-
-template <typename T>
-__device__ __forceinline__ float load_x(const T* p, int i);
-template <>
-__device__ __forceinline__ float load_x<float>(const float* p, int i)
-{
-    return __ldcs(p + i);  // read once: evict first, the tile rings stay in L2
-}
-template <>
-__device__ __forceinline__ float load_x<uint16_t>(const uint16_t* p, int i)
-{
-    return bf16_to_f32(__ldcs((const unsigned short*)p + i));
-}
+__host__ __device__ constexpr int enc_smem_bytes(int U) { return NWARPS * 2 * GBUF + enc_wb_bytes(U); }
+// Of a decoder CTA: two group buffers per warp.
+constexpr int DEC_SMEM_BYTES = NWARPS * 2 * GBUF;
+constexpr int DEC_CTAS_PER_SM = 3;
 
 __device__ __forceinline__ void store_raw(void* p, int dtype, unsigned long long i, float v)
 {
@@ -224,173 +199,7 @@ __device__ __forceinline__ int check_header(const Item& it, Ctl* ctl, unsigned i
 __device__ __forceinline__ int planes_of(int w) { return w ? w + 1 : 0; }
 
 
-__device__ __forceinline__ uint8_t width_byte(int np) { return (uint8_t)(np ? np - 1 : 0); }
-
-// width_byte of four blocks at once, from their plane counts packed one per
-// byte (each at most 32).  Adding 0x7f to a byte sets its top bit exactly when
-// its count is nonzero and carries into no neighbour, so subtracting those
-// bits, shifted down to bit 0, borrows across no byte.
-__device__ __forceinline__ uint32_t width_bytes4(uint32_t c)
-{
-    return c - (((c + 0x7f7f7f7fu) & 0x80808080u) >> 7);
-}
-
-// Inclusive prefix sum of exact FP32 integers over 32 lanes (FMA pipe).
-__device__ __forceinline__ float scan_incl_f(float v)
-{
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        asm("{\n\t.reg .f32 t;\n\t.reg .pred p;\n\t"
-            "shfl.sync.up.b32 t|p, %0, %1, 0, -1;\n\t"
-            "@p add.rn.f32 %0, %0, t;\n\t}"
-            : "+f"(v)
-            : "r"(off));
-    }
-    return v;
-}
-// The same over segments of 16 lanes.
-__device__ __forceinline__ float scan_incl_f16(float v)
-{
-#pragma unroll
-    for (int off = 1; off < 16; off <<= 1) {
-        asm("{\n\t.reg .f32 t;\n\t.reg .pred p;\n\t"
-            "shfl.sync.up.b32 t|p, %0, %1, 4096, -1;\n\t"
-            "@p add.rn.f32 %0, %0, t;\n\t}"
-            : "+f"(v)
-            : "r"(off));
-    }
-    return v;
-}
-
-// ---- decoding ------------------------------------------------------------------
-// Two rows' sign-magnitude words u_a | u_b << 16 (each below 2^11: |d| <=
-// 1023) -> d_a + B | (d_b + B) << 16 with B = 1024: both halves in [1, 2047],
-// so an integer prefix sum over 32 lanes (at most 65504 per half) carries
-// nothing from one half into the other and two rows scan with one shuffle per
-// step.  Sum at lane j: q_j - q_-1 + (j + 1) B, q_-1 the value before the row.
-constexpr uint32_t PAIR_B = 1024u;
-constexpr int PAIR_MAX_PLANES = 11;
-__device__ __forceinline__ uint32_t biased_pair(uint32_t t)
-{
-    const uint32_t m2 = (t >> 1) & 0x7fff7fffu;                  // magnitudes
-    const uint32_t plus = (PAIR_B | PAIR_B << 16) + m2;
-    const uint32_t minus = (PAIR_B | PAIR_B << 16) - m2;         // no borrow: each half >= 1
-    const uint32_t neg = (t & 0x00010001u) * 0xffffu;            // all-ones halves where d < 0
-    return (plus & ~neg) | (minus & neg);
-}
-// Exact FP32 of a half of a biased pair scan: (half + kbits) holds the float
-// bits of q + 1.5 * 2^23 (|q| < 2^22), kbits = 0x4b400000 - (j + 1) B (+ the
-// value before the row when it is nonzero, added by the caller in FP32).
-__device__ __forceinline__ float pair_half_f(uint32_t half, uint32_t kbits)
-{
-    return __fsub_rn(__uint_as_float(half + kbits), 12582912.0f);
-}
-
-// Block planes and payload offsets of one warp unit of an input stream:
-// meta[b] = (planes, byte offset from the unit's payload start) for the
-// unit's blocks.  Returns the unit's payload start in the stream; a unit whose
-// planes would lie beyond cin_cap is reported and gets zero planes.
-// off_local >= 0: the unit's payload offset found by the caller (a small
-// item's decoder CTA), in place of the width scan's P.offs[slot].
-template <int LOG2L, int U, bool HEADS = false>
-__device__ __forceinline__ unsigned long long unit_meta(const Launch& P, const Item& it,
-                                                        unsigned slot, unsigned long long ue0,
-                                                        int2* meta, bool& narrow, bool& narrow11,
-                                                        long long off_local = -1)
-{
-    constexpr int L = 1 << LOG2L;
-    constexpr int PB = L / 8;
-    constexpr int BU = U * 32 / L;                // blocks per unit
-    constexpr int BPL = BU >= 32 ? BU / 32 : 1;   // blocks per lane
-    const int lane = threadIdx.x & 31;
-    const unsigned long long nb = (it.n + L - 1) >> LOG2L;
-    const unsigned long long b0 = (ue0 >> LOG2L) + (unsigned long long)lane * BPL;
-    static_assert(BPL == 1 || BPL == 2 || BPL == 4 || BPL == 8, "width bytes per lane");
-    const bool mine = BU >= 32 || lane < BU;
-    uint32_t wv[2] = {0u, 0u};  // this lane's BPL width bytes, little-endian
-    if (mine && b0 < ceil16(nb)) {
-        // b0 is a multiple of BPL and the width bytes are zero padded to 16:
-        // the BPL bytes from b0 are inside the stream and naturally aligned
-        const uint8_t* wp = it.cin + 32 + b0;
-        if (BPL == 8) {
-            const uint2 v = __ldg((const uint2*)wp);
-            wv[0] = v.x;
-            wv[1] = v.y;
-        } else if (BPL == 4) {
-            wv[0] = __ldg((const unsigned*)wp);
-        } else if (BPL == 2) {
-            wv[0] = __ldg((const unsigned short*)wp);
-        } else {
-            wv[0] = __ldg(wp);
-        }
-    }
-    int np[BPL];
-    int sum = 0;
-    bool bad = false;
-#pragma unroll
-    for (int i = 0; i < BPL; ++i) {
-        int w = (wv[i >> 2] >> (8 * (i & 3))) & 0xff;
-        if (w > ZC_MAX_WIDTH) {
-            bad = true;
-            w = 0;
-        }
-        np[i] = planes_of(w);
-        sum += np[i] * PB;
-    }
-    if (bad) fail(P.ctl, ZC_ERR_FORMAT, b0);
-    {
-        int npmax = 0;
-#pragma unroll
-        for (int i = 0; i < BPL; ++i) npmax = max(npmax, np[i]);
-        narrow = __all_sync(FULL, npmax <= 16);
-        narrow11 = !HEADS && __all_sync(FULL, npmax <= PAIR_MAX_PLANES);
-    }
-    int tot;
-    int off = warp_excl_scan(sum, lane, tot);
-    const bool slot_ok = off_local >= 0 || dcheck(P.ctl, slot < P.ws_cap, slot);
-    const unsigned long long uoff =
-        off_local >= 0 ? (unsigned long long)off_local : (slot_ok ? P.offs[slot] : 0ull);
-    const unsigned long long base = 32ull + ceil16(nb) + (HEADS ? ceil16(3ull * nb) : 0ull) + uoff;
-    const bool ok = slot_ok && base + (unsigned long long)tot <= it.cin_cap;
-    if (!ok && lane == 0) fail(P.ctl, ZC_ERR_FORMAT, slot);
-    if (DEBUG_BUILD && mine && lane == (BU >= 32 ? 31 : BU - 1))
-        dcheck(P.ctl, off + sum == tot, slot);  // the last block's planes end at the unit's
-    __syncwarp();  // earlier readers of meta are done
-    if (mine) {
-#pragma unroll
-        for (int i = 0; i < BPL; ++i) {
-            meta[lane * BPL + i] = make_int2(ok ? np[i] : 0, off);
-            off += np[i] * PB;
-        }
-    }
-    __syncwarp();
-    // the whole unit payload is requested into L2 at once (one bulk prefetch,
-    // 16-byte aligned inner range); the per-group plane loads then hit L2
-    if (ok && lane == 0 && tot > 0) {
-        const uintptr_t a0 = (uintptr_t)(it.cin + base), a1 = a0 + (uintptr_t)tot;
-        const uintptr_t s0 = (a0 + 15) & ~(uintptr_t)15, s1 = a1 & ~(uintptr_t)15;
-        if (s1 > s0)
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(s0),
-                         "r"((unsigned)(s1 - s0))
-                         : "memory");
-    }
-    return ok ? base : 0ull;
-}
-
-// Sign-magnitude word of one element -> its delta as an exact FP32 value
-// (|d| < 2^23), the sign injected into the float's sign bit.
-__device__ __forceinline__ float delta_f(uint32_t u)
-{
-    const float mag = __fsub_rn(__int_as_float((u >> 1) | 0x4b000000u), 8388608.0f);
-    return __int_as_float(__float_as_int(mag) ^ (u << 31));
-}
-
-// Decodes rows [g GR, g GR + GR) of a warp unit into acc[] (x^ = q * 2eb).
-// `src` points at the unit's payload, `meta` at its block metadata.  All of
-// the group's plane words are requested before the first transpose so their
-// loads overlap.  A pair of rows whose blocks have at most 16 planes shares
-// one transpose and is scanned in FP32 (every partial sum is an integer below
-// 2^22: exact); wider rows are scanned in integers.
+// ---- stream access ------------------------------------------------------------
 // Block head of the heads-apart format: 24-bit two's complement, little-endian.
 __device__ __forceinline__ int load_head(const uint8_t* p)
 {
@@ -399,506 +208,29 @@ __device__ __forceinline__ int load_head(const uint8_t* p)
     return (int)v - ((v & 0x800000u) ? (1 << 24) : 0);
 }
 
-template <int LOG2L, bool NARROW, bool HEADS = false, bool BIASED = false>
-__device__ __forceinline__ void decode_group(const uint8_t* src, const int2* meta, int g,
-                                             float two_eb, float acc[GR], const TpC& tc,
-                                             const uint8_t* hsrc = nullptr)
+// Width byte(s) of this lane's row of the group whose first block is bg (a
+// multiple of 8; L = 16: the two bytes of the row's blocks).  The width bytes
+// are zero padded to 16, blocks beyond them have none.
+template <int LOG2L>
+__device__ __forceinline__ uint32_t load_widths(const uint8_t* cin, unsigned long long nb,
+                                                unsigned long long bg)
 {
-    constexpr int L = 1 << LOG2L;
-    constexpr int RPB = L >= 32 ? L / 32 : 1;
-    constexpr int NR = L == 128 ? 4 : 2;  // rows per step (pair, or quad at L = 128)
-    constexpr int NS = GR / NR;           // steps per group
     const int lane = threadIdx.x & 31;
-    const int k = lane & 15;
-    const bool hi = lane >= 16;
-    const int fb = L >= 32 ? g * GR / RPB : g * GR * 2;  // first block of the group
-    const int2* mt = meta + fb;
-    // ---- phase 1: metadata, plane loads (and block heads) of every step ----
-    int hv[GR];  // heads apart: the head of this lane's block where this lane is one
-    if (HEADS) {
-#pragma unroll
-        for (int r = 0; r < GR; ++r) {
-            hv[r] = 0;
-            int b = -1;  // block of the unit whose head this lane holds in row r
-            if (L == 16 && k == 0) b = 2 * (g * GR + r) + (hi ? 1 : 0);
-            else if (L == 32 && lane == 0) b = g * GR + r;
-            else if (L >= 64 && lane == 0 && (r % RPB) == 0) b = (g * GR + r) / RPB;
-            if (b >= 0) hv[r] = load_head(hsrc + 3 * b);
-        }
-    }
-    uint32_t wv[NS][NR];
-    unsigned paired = 0;  // bit s: step s has at most 16 planes per block
-    static_assert(!BIASED || (NARROW && !HEADS), "the biased pair scan: narrow plain units");
-#pragma unroll
-    for (int st = 0; st < NS; ++st) {
-        const int r = st * NR;
-        if (L == 32) {
-            const int4 m = *(const int4*)&mt[r];
-            if (NARROW || (m.x <= 16 && m.z <= 16)) {
-                paired |= 1u << st;
-                const int np = hi ? m.z : m.x, off = hi ? m.w : m.y;
-                wv[st][0] = k < np ? __ldg((const unsigned*)src + (((unsigned)off >> 2) + k)) : 0u;
-            } else {
-                wv[st][0] = lane < m.x ? __ldg((const unsigned*)(src + m.y) + lane) : 0u;
-                wv[st][1] = lane < m.z ? __ldg((const unsigned*)(src + m.w) + lane) : 0u;
-            }
-        } else if (L == 16) {
-            const int4 m0 = *(const int4*)&mt[2 * r];
-            const int4 m1 = *(const int4*)&mt[2 * r + 2];
-            if (NARROW || max(max(m0.x, m0.z), max(m1.x, m1.z)) <= 16) {
-                paired |= 1u << st;
-                const int npL = hi ? m1.x : m0.x, offL = hi ? m1.y : m0.y;
-                const int npH = hi ? m1.z : m0.z, offH = hi ? m1.w : m0.w;
-                const uint32_t wl = k < npL ? __ldg((const unsigned short*)(src + offL) + k) : 0u;
-                const uint32_t wh = k < npH ? __ldg((const unsigned short*)(src + offH) + k) : 0u;
-                wv[st][0] = wl | (wh << 16);
-            } else {
-                uint32_t wl = lane < m0.x ? __ldg((const unsigned short*)(src + m0.y) + lane) : 0u;
-                uint32_t wh = lane < m0.z ? __ldg((const unsigned short*)(src + m0.w) + lane) : 0u;
-                wv[st][0] = wl | (wh << 16);
-                wl = lane < m1.x ? __ldg((const unsigned short*)(src + m1.y) + lane) : 0u;
-                wh = lane < m1.z ? __ldg((const unsigned short*)(src + m1.w) + lane) : 0u;
-                wv[st][1] = wl | (wh << 16);
-            }
-        } else if (L == 64) {
-            const int2 m = mt[r / 2];
-            if (NARROW || m.x <= 16) {
-                paired |= 1u << st;
-                wv[st][0] =
-                    k < m.x ? __ldg((const unsigned*)(src + m.y + 8 * k + (hi ? 4 : 0))) : 0u;
-            } else {
-                uint2 v = make_uint2(0u, 0u);
-                if (lane < m.x) v = __ldg((const uint2*)(src + m.y) + lane);
-                wv[st][0] = v.x;
-                wv[st][1] = v.y;
-            }
-        } else {
-            const int2 m = mt[r / 4];
-            if (NARROW || m.x <= 16) {
-                paired |= 1u << st;
-                const uint8_t* pp = src + m.y + 16 * k + (hi ? 4 : 0);
-                wv[st][0] = k < m.x ? __ldg((const unsigned*)pp) : 0u;
-                wv[st][1] = k < m.x ? __ldg((const unsigned*)(pp + 8)) : 0u;
-            } else {
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (lane < m.x) v = __ldg((const uint4*)(src + m.y) + lane);
-                wv[st][0] = v.x;
-                wv[st][1] = v.y;
-                wv[st][2 % NR] = v.z;
-                wv[st][3 % NR] = v.w;
-            }
-        }
-    }
-    // ---- phase 2: transposes, prefix sums, reconstruction ----
-#pragma unroll
-    for (int st = 0; st < NS; ++st) {
-        const int r = st * NR;
-        if (BIASED) {
-            // lane position within its block row
-            const uint32_t kbits = 0x4b400000u - ((uint32_t)(L == 16 ? k : lane) + 1u) * PAIR_B;
-            // two rows per integer scan: (q + (j + 1) B) of both rows in one word
-            float carry = 0.0f;
-#pragma unroll
-            for (int h2 = 0; h2 < NR; h2 += 2) {
-                uint32_t v = biased_pair(tpose(wv[st][h2 / 2], tc));
-                v = (uint32_t)(L == 16 ? scan_incl<16>((int)v) : scan_incl<32>((int)v));
-                float fa = pair_half_f(v & 0xffffu, kbits);
-                float fb = pair_half_f(v >> 16, kbits);
-                if (L >= 64) {
-                    // rows of one block: each continues from the last value of the row before
-                    if (((r + h2) % RPB) != 0) fa = __fadd_rn(fa, carry);
-                    fb = __fadd_rn(fb, __shfl_sync(FULL, fa, 31));
-                    if (((r + h2 + 1) % RPB) != RPB - 1) carry = __shfl_sync(FULL, fb, 31);
-                }
-                acc[r + h2] = __fmul_rn(fa, two_eb);
-                acc[r + h2 + 1] = __fmul_rn(fb, two_eb);
-            }
-            continue;
-        }
-        uint32_t u[4];
-        const bool pr = NARROW || ((paired >> st) & 1u);
-        if (pr) {
-            const uint32_t t0 = tpose(wv[st][0], tc);
-            u[0] = t0 & 0xffffu;
-            u[1] = t0 >> 16;
-            if (NR == 4) {
-                const uint32_t t1 = tpose(wv[st][1 % NR], tc);
-                u[2] = t1 & 0xffffu;
-                u[3] = t1 >> 16;
-            }
-        } else {
-#pragma unroll
-            for (int h = 0; h < NR; ++h) u[h] = tpose(wv[st][h], tc);
-        }
-        if (pr) {
-            float carry = 0.0f;
-#pragma unroll
-            for (int h = 0; h < NR; ++h) {
-                float dv = delta_f(u[h]);
-                if (HEADS) dv = __fadd_rn(dv, __int2float_rn(hv[r + h]));  // the head's delta is 0
-                float v = L == 16 ? scan_incl_f16(dv) : scan_incl_f(dv);
-                if (L >= 64 && ((r + h) % RPB) != 0) v = __fadd_rn(v, carry);
-                if (L >= 64 && ((r + h) % RPB) != RPB - 1) carry = __shfl_sync(FULL, v, 31);
-                acc[r + h] = __fmul_rn(v, two_eb);
-            }
-        } else {
-            int carry = 0;
-#pragma unroll
-            for (int h = 0; h < NR; ++h) {
-                const int mag = (int)(u[h] >> 1);
-                int dv = (u[h] & 1u) ? -mag : mag;
-                if (HEADS) dv += hv[r + h];
-                int v = L == 16 ? scan_incl<16>(dv) : scan_incl<32>(dv);
-                if (L >= 64 && ((r + h) % RPB) != 0) v += carry;
-                if (L >= 64 && ((r + h) % RPB) != RPB - 1) carry = __shfl_sync(FULL, v, 31);
-                acc[r + h] = __fmul_rn(__int2float_rn(v), two_eb);
-            }
-        }
-    }
+    const unsigned long long b =
+        bg + (LOG2L == 4 ? 2u * lane : LOG2L == 5 ? lane : LOG2L == 6 ? lane / 2 : lane / 4);
+    if (b >= ceil16(nb)) return 0u;
+    return LOG2L == 4 ? (uint32_t)__ldg((const unsigned short*)(cin + 32 + b))
+                      : (uint32_t)__ldg(cin + 32 + b);
 }
 
-// ---- encoding ------------------------------------------------------------------
-// Predicated stores without a branch: the store happens when a < b.  `p` is
-// a shared-memory address (the warp's staging buffer).
-__device__ __forceinline__ void sts_u32_if(unsigned p, uint32_t v, int a, int b)
+// Requests [p, p + len) into L2 (one bulk prefetch of the 16-byte aligned inner range).
+__device__ __forceinline__ void prefetch_l2(const void* p, unsigned len)
 {
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.s32 q, %2, %3;\n\t@q st.shared.u32 [%0], %1;\n\t}"
-                 ::"r"(p), "r"(v), "r"(a), "r"(b) : "memory");
-}
-__device__ __forceinline__ void sts_u16_if(unsigned p, uint32_t v, int a, int b)
-{
-    asm volatile("{\n\t.reg .pred q;\n\t.reg .b16 h;\n\tcvt.u16.u32 h, %1;\n\t"
-                 "setp.lt.s32 q, %2, %3;\n\t@q st.shared.u16 [%0], h;\n\t}"
-                 ::"r"(p), "r"(v), "r"(a), "r"(b) : "memory");
-}
-__device__ __forceinline__ void sts_u64_if(unsigned p, uint32_t v0, uint32_t v1, int a, int b)
-{
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.s32 q, %3, %4;\n\t@q st.shared.v2.u32 [%0], {%1, %2};\n\t}"
-                 ::"r"(p), "r"(v0), "r"(v1), "r"(a), "r"(b) : "memory");
-}
-__device__ __forceinline__ void sts_u128_if(unsigned p, uint32_t v0, uint32_t v1, uint32_t v2,
-                                            uint32_t v3, int a, int b)
-{
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.s32 q, %5, %6;\n\t"
-                 "@q st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n\t}"
-                 ::"r"(p), "r"(v0), "r"(v1), "r"(v2), "r"(v3), "r"(a), "r"(b) : "memory");
-}
-// Stores when m != 0 (a lane's bit of a mask); `p` is a shared-memory address.
-__device__ __forceinline__ void sts_u32_m(unsigned p, uint32_t v, uint32_t m)
-{
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.shared.u32 [%0], %1;\n\t}"
-                 ::"r"(p), "r"(v), "r"(m) : "memory");
-}
-__device__ __forceinline__ void sts_u8_m(unsigned p, uint32_t v, uint32_t m)
-{
-    asm volatile("{\n\t.reg .pred q;\n\t.reg .b16 h;\n\tcvt.u16.u32 h, %1;\n\t"
-                 "setp.ne.u32 q, %2, 0;\n\t@q st.shared.u8 [%0], h;\n\t}"
-                 ::"r"(p), "r"(v), "r"(m) : "memory");
-}
-__device__ __forceinline__ uint32_t lanemask_lt()
-{
-    uint32_t m;
-    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
-    return m;
-}
-// Predicated shared-memory stores of width bytes (`p` in shared memory).
-__device__ __forceinline__ void sts_if(uint8_t* p, uint4 v, bool c)
-{
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %5, 0;\n\t@q st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n\t}"
-                 ::"r"((unsigned)__cvta_generic_to_shared(p)), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"((int)c) : "memory");
-}
-__device__ __forceinline__ void sts_if(uint8_t* p, uint2 v, bool c)
-{
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %3, 0;\n\t@q st.shared.v2.u32 [%0], {%1, %2};\n\t}"
-                 ::"r"((unsigned)__cvta_generic_to_shared(p)), "r"(v.x), "r"(v.y), "r"((int)c) : "memory");
-}
-__device__ __forceinline__ void sts_if(uint8_t* p, uint32_t v, bool c)
-{
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\t@q st.shared.u32 [%0], %1;\n\t}"
-                 ::"r"((unsigned)__cvta_generic_to_shared(p)), "r"(v), "r"((int)c) : "memory");
-}
-__device__ __forceinline__ void sts_if(uint8_t* p, unsigned short v, bool c)
-{
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\t@q st.shared.u16 [%0], %1;\n\t}"
-                 ::"r"((unsigned)__cvta_generic_to_shared(p)), "h"(v), "r"((int)c) : "memory");
-}
-
-// The previous lane's q within segments of W lanes; the first lane of a
-// segment gets `fill` (uses the in-range predicate of shfl.up).
-template <int W>
-__device__ __forceinline__ int prev_lane(int q, int fill)
-{
-    int p;
-    asm("{\n\t.reg .pred ok;\n\t"
-        "shfl.sync.up.b32 %0|ok, %1, 1, %2, -1;\n\t"
-        "@!ok mov.b32 %0, %3;\n\t}"
-        : "=r"(p)
-        : "r"(q), "r"((32 - W) << 8), "r"(fill));
-    return p;
-}
-
-// Quantizes, delta-codes and bit-plane packs GR rows (the first `nrem`
-// elements are valid, all of them when ALL; the rest are padding with zero
-// deltas), appends the planes of their blocks at byte `lo` of the unit's
-// payload (shared-memory address seg + lo: the warp's staging buffer), writes
-// their width bytes to `wb` (shared memory, one store per group), ORs any
-// quantizer error into `err`, and returns the new `lo`.  Two rows whose
-// values fit 16 bits share one transpose.
-template <int LOG2L, bool ALL, bool HEADS = false>
-__device__ __forceinline__ int encode_group(const float acc[GR], int nrem, float eb, float two_eb,
-                                            float inv, unsigned seg, int lo, uint8_t* wb, int& err,
-                                            const TpC& tc, uint8_t* hout = nullptr)
-{
-    constexpr int L = 1 << LOG2L;
-    constexpr int RPB = L >= 32 ? L / 32 : 1;
-    const int lane = threadIdx.x & 31;
-    const int k = lane & 15;
-    const bool hi = lane >= 16;
-    // quantize: the exactness of the fast rounding is voted once per group.
-    // q holds q + QBIAS (the rounded float's bits): the deltas are the same
-    int q[GR];
-    {
-        bool slow = false;
-#pragma unroll
-        for (int r = 0; r < GR; ++r) slow |= !quantize_fast_bits(acc[r], inv, q[r]);
-        if (__any_sync(FULL, slow)) {
-#pragma unroll
-            for (int r = 0; r < GR; ++r) {
-                int qq = 0;
-                if (ALL || r * 32 + lane < nrem) err |= quantize(acc[r], eb, two_eb, inv, qq);
-                q[r] = qq + QBIAS;
-            }
-        }
-    }
-    uint32_t u[GR];
-    uint32_t wide = 0;
-    int carry = 0;
-#pragma unroll
-    for (int r = 0; r < GR; ++r) {
-        const int fill = (L >= 64 && (r % RPB) != 0) ? carry : QBIAS;  // a block starts from q = 0
-        const int prev = prev_lane<L == 16 ? 16 : 32>(q[r], fill);
-        if (L >= 64 && (r % RPB) != RPB - 1) carry = __shfl_sync(FULL, q[r], 31);
-        int d = q[r] - prev;
-        if (!ALL && r * 32 + lane >= nrem) d = 0;
-        if (HEADS) {
-            // heads apart: the block head goes to its 3-byte field (in the
-            // output, at block position), its own delta is 0
-            int b = -1;
-            if (L == 16 && k == 0) b = 2 * r + (hi ? 1 : 0);
-            else if (L == 32 && lane == 0) b = r;
-            else if (L >= 64 && lane == 0 && (r % RPB) == 0) b = r / RPB;
-            if (b >= 0) {
-                if (ALL || r * 32 + lane < nrem) {
-                    const int head = q[r] - QBIAS;
-                    uint8_t* p = hout + 3 * b;
-                    p[0] = (uint8_t)head;
-                    p[1] = (uint8_t)(head >> 8);
-                    p[2] = (uint8_t)(head >> 16);
-                }
-                d = 0;
-            }
-        }
-        const uint32_t ad = (uint32_t)(d < 0 ? -d : d);
-        u[r] = __funnelshift_l((uint32_t)d, ad, 1);  // |d| << 1 | sign
-        wide |= u[r];
-    }
-    // one vote: does any value of the group need more than 16 planes?
-    const bool any_wide = __any_sync(FULL, (wide >> 16) != 0u);
-    const uint32_t hmask = hi ? 0xffffffffu : 0u;
-    // the group's width bytes, gathered in registers and stored once (GR * 32 / L bytes)
-    uint32_t wacc[4] = {0u, 0u, 0u, 0u};
-    uint32_t pk[GR / 2];  // L = 32: plane counts of the row pairs
-    // Every value of the group within 8 planes (the common case at moderate
-    // bounds; L >= 32): four rows share a transpose, and lane 8m + j then
-    // holds plane j of row m.  M is the ballot of nonzero planes.
-    //   L = 32 (a block per row): smearing every byte of M downwards gives F,
-    //   whose byte m has the low np_m bits set; a lane stores its plane if
-    //   its bit of F is set, at 4 popc(F & lanes below) bytes past the quad's
-    //   start, and the quad takes 4 popc(F) bytes.  The lane at a row's top
-    //   plane (j = np - 1), or lane j = 0 of a row without planes, writes the
-    //   row's width byte, j, itself.
-    //   L = 64 (rows 0-1 and 2-3 are blocks): the block masks are bytes 0 | 1
-    //   and 2 | 3 of M; plane j of a block is 8 bytes, its two rows' words.
-    //   L = 128 (one block): the block mask is the OR of M's bytes; plane j
-    //   is 16 bytes, the four rows' words.
-    const bool quad = L >= 32 && !any_wide && !__any_sync(FULL, (wide >> 8) != 0u);
-    if (quad) {
-        const int j = lane & 7, m4 = lane >> 3;
-        const uint32_t lt = lanemask_lt(), eq = 1u << lane;
-        const unsigned wrow = (unsigned)__cvta_generic_to_shared(wb) + (unsigned)m4;
-#pragma unroll
-        for (int r = 0; r < GR; r += 4) {
-            const uint32_t w = __byte_perm(__byte_perm(u[r], u[r + 1], 0x0040),
-                                           __byte_perm(u[r + 2], u[r + 3], 0x0040), 0x5410);
-            const uint32_t t = tpose(w, tc);
-            const uint32_t M = __ballot_sync(FULL, t != 0u);
-            if (L == 32) {
-                uint32_t F = M | ((M >> 1) & 0x7f7f7f7fu);
-                F |= (F >> 2) & 0x3f3f3f3fu;
-                F |= (F >> 4) & 0x0f0f0f0fu;
-                sts_u32_m(seg + lo + 4u * (unsigned)__popc(F & lt), t, F & eq);
-                const uint32_t top = (F & ~((F >> 1) & 0x7f7f7f7fu)) | (~F & 0x01010101u);
-                sts_u8_m(wrow + r, (uint32_t)j, top & eq);
-                lo += 4 * __popc(F);
-            } else if (L == 64) {
-                const uint32_t X = M | (M >> 8);
-                const int npA = 32 - __clz(X & 0xffu), npB = 32 - __clz((X >> 16) & 0xffu);
-                sts_u32_if(seg + lo + 8 * j + 4 * (m4 & 1) + (hmask & (8 * npA)), t, j,
-                           hi ? npB : npA);
-                wacc[0] |= ((uint32_t)width_byte(npA) | ((uint32_t)width_byte(npB) << 8)) << (8 * (r / 2));
-                lo += 8 * (npA + npB);
-            } else {
-                const uint32_t X = M | (M >> 16);
-                const int np = 32 - __clz((X | (X >> 8)) & 0xffu);
-                sts_u32_if(seg + lo + 16 * j + 4 * m4, t, j, np);
-                wacc[0] |= (uint32_t)width_byte(np) << (8 * (r / 4));
-                lo += 16 * np;
-            }
-        }
-    } else if (!any_wide) {
-        // every value of the group fits 16 bits (the common case): paired (or
-        // quadrupled) rows share a transpose, with no per-pair votes
-#pragma unroll
-        for (int r = 0; r < GR; r += (L == 128 ? 4 : 2)) {
-            if (L == 32) {
-                const uint32_t t = tpose(__byte_perm(u[r], u[r + 1], 0x5410), tc);
-                const unsigned m = __ballot_sync(FULL, t != 0u);
-                const int na = 32 - __clz(m & 0xffffu), nb = 32 - __clz(m >> 16);
-                sts_u32_if(seg + 4 * k + lo + (hmask & (4 * na)), t, k, hi ? nb : na);
-                // the pair's plane counts as bytes [na, nb, 0, 0]
-                pk[r / 2] = __byte_perm((uint32_t)na, (uint32_t)nb, 0x1140);
-                lo += 4 * (na + nb);
-            } else if (L == 16) {
-                const uint32_t t = tpose(__byte_perm(u[r], u[r + 1], 0x5410), tc);
-                const unsigned m0 = __ballot_sync(FULL, (t & 0xffffu) != 0u);
-                const unsigned m1 = __ballot_sync(FULL, (t >> 16) != 0u);
-                const int npA = 32 - __clz(m0 & 0xffffu), npB = 32 - __clz(m1 & 0xffffu);
-                const int npC = 32 - __clz(m0 >> 16), npD = 32 - __clz(m1 >> 16);
-                const int oA = lo, oB = oA + 2 * npA, oC = oB + 2 * npB, oD = oC + 2 * npC;
-                sts_u16_if(seg + (hi ? oC : oA) + 2 * k, t & 0xffffu, k, hi ? npC : npA);
-                sts_u16_if(seg + (hi ? oD : oB) + 2 * k, t >> 16, k, hi ? npD : npB);
-                wacc[r / 2] = (uint32_t)width_byte(npA) | ((uint32_t)width_byte(npB) << 8) |
-                              ((uint32_t)width_byte(npC) << 16) | ((uint32_t)width_byte(npD) << 24);
-                lo += 2 * (npA + npB + npC + npD);
-            } else if (L == 64) {
-                const uint32_t t = tpose(__byte_perm(u[r], u[r + 1], 0x5410), tc);
-                const unsigned m = __ballot_sync(FULL, t != 0u);
-                const int np = 32 - __clz((m & 0xffffu) | (m >> 16));
-                sts_u32_if(seg + lo + 8 * k + (hmask & 4), t, k, np);
-                wacc[0] |= (uint32_t)width_byte(np) << (8 * (r / 2));
-                lo += 8 * np;
-            } else {
-                const uint32_t t0 = tpose(__byte_perm(u[r], u[r + 1], 0x5410), tc);
-                const uint32_t t1 = tpose(__byte_perm(u[r + 2], u[r + 3], 0x5410), tc);
-                const unsigned m = __ballot_sync(FULL, (t0 | t1) != 0u);
-                const int np = 32 - __clz((m & 0xffffu) | (m >> 16));
-                const unsigned pp = seg + lo + 16 * k + (hmask & 4);
-                sts_u32_if(pp, t0, k, np);
-                sts_u32_if(pp + 8, t1, k, np);
-                wacc[0] |= (uint32_t)width_byte(np) << (8 * (r / 4));
-                lo += 16 * np;
-            }
-        }
-        if (L == 32) {
-            // the width bytes of two pairs at a time
-#pragma unroll
-            for (int w = 0; w < GR / 4; ++w)
-                wacc[w] = width_bytes4(__byte_perm(pk[2 * w], pk[2 * w + 1], 0x5410));
-        }
-    } else {
-    #pragma unroll
-        for (int r = 0; r < GR; r += (L == 128 ? 4 : 2)) {
-            if (L == 32) {
-                int fa, fb;  // highest nonzero plane of blocks r, r + 1 (-1: none)
-                if (!any_wide || !__any_sync(FULL, ((u[r] | u[r + 1]) >> 16) != 0u)) {
-                    const uint32_t t = tpose(__byte_perm(u[r], u[r + 1], 0x5410), tc);
-                    const unsigned m = __ballot_sync(FULL, t != 0u);
-                    fa = 31 - __clz(m & 0xffffu);
-                    fb = 31 - __clz(m >> 16);
-                    const int npm = hi ? fb + 1 : fa + 1;
-                    sts_u32_if(seg + lo + (hmask & (4 * fa + 4)) + 4 * k, t, k, npm);
-                } else {
-                    const uint32_t ta = tpose(u[r], tc), tb = tpose(u[r + 1], tc);
-                    fa = 31 - __clz(__ballot_sync(FULL, ta != 0u));
-                    fb = 31 - __clz(__ballot_sync(FULL, tb != 0u));
-                    sts_u32_if(seg + lo + 4 * lane, ta, lane, fa + 1);
-                    sts_u32_if(seg + lo + 4 * fa + 4 + 4 * lane, tb, lane, fb + 1);
-                }
-                wacc[r / 4] |= ((uint32_t)max(fa, 0) | ((uint32_t)max(fb, 0) << 8)) << (8 * (r % 4));
-                lo += 4 * (fa + fb + 2);
-            } else if (L == 16) {
-                int npA, npB, npC, npD;
-                if (!any_wide || !__any_sync(FULL, ((u[r] | u[r + 1]) >> 16) != 0u)) {
-                    const uint32_t t = tpose(__byte_perm(u[r], u[r + 1], 0x5410), tc);
-                    const unsigned m0 = __ballot_sync(FULL, (t & 0xffffu) != 0u);
-                    const unsigned m1 = __ballot_sync(FULL, (t >> 16) != 0u);
-                    npA = 32 - __clz(m0 & 0xffffu);
-                    npB = 32 - __clz(m1 & 0xffffu);
-                    npC = 32 - __clz(m0 >> 16);
-                    npD = 32 - __clz(m1 >> 16);
-                    const int oA = lo, oB = oA + 2 * npA, oC = oB + 2 * npB, oD = oC + 2 * npC;
-                    const int npL = hi ? npC : npA, npH = hi ? npD : npB;
-                    const int offL = hi ? oC : oA, offH = hi ? oD : oB;
-                    sts_u16_if(seg + offL + 2 * k, t & 0xffffu, k, npL);
-                    sts_u16_if(seg + offH + 2 * k, t >> 16, k, npH);
-                } else {
-                    const uint32_t ta = tpose(u[r], tc), tb = tpose(u[r + 1], tc);
-                    npA = 32 - __clz(__ballot_sync(FULL, (ta & 0xffffu) != 0u));
-                    npB = 32 - __clz(__ballot_sync(FULL, (ta >> 16) != 0u));
-                    npC = 32 - __clz(__ballot_sync(FULL, (tb & 0xffffu) != 0u));
-                    npD = 32 - __clz(__ballot_sync(FULL, (tb >> 16) != 0u));
-                    const int oA = lo, oB = oA + 2 * npA, oC = oB + 2 * npB, oD = oC + 2 * npC;
-                    sts_u16_if(seg + oA + 2 * lane, ta & 0xffffu, lane, npA);
-                    sts_u16_if(seg + oB + 2 * lane, ta >> 16, lane, npB);
-                    sts_u16_if(seg + oC + 2 * lane, tb & 0xffffu, lane, npC);
-                    sts_u16_if(seg + oD + 2 * lane, tb >> 16, lane, npD);
-                }
-                wacc[r / 2] = (uint32_t)width_byte(npA) | ((uint32_t)width_byte(npB) << 8) |
-                              ((uint32_t)width_byte(npC) << 16) | ((uint32_t)width_byte(npD) << 24);
-                lo += 2 * (npA + npB + npC + npD);
-            } else if (L == 64) {
-                int np;
-                if (!any_wide || !__any_sync(FULL, ((u[r] | u[r + 1]) >> 16) != 0u)) {
-                    const uint32_t t = tpose(__byte_perm(u[r], u[r + 1], 0x5410), tc);
-                    const unsigned m = __ballot_sync(FULL, t != 0u);
-                    np = 32 - __clz((m & 0xffffu) | (m >> 16));
-                    sts_u32_if(seg + lo + 8 * k + (hmask & 4), t, k, np);
-                } else {
-                    const uint32_t ta = tpose(u[r], tc), tb = tpose(u[r + 1], tc);
-                    np = 32 - __clz(__ballot_sync(FULL, (ta | tb) != 0u));
-                    sts_u64_if(seg + lo + 8 * lane, ta, tb, lane, np);
-                }
-                wacc[0] |= (uint32_t)width_byte(np) << (8 * (r / 2));
-                lo += 8 * np;
-            } else {
-                int np;
-                if (!any_wide ||
-                    !__any_sync(FULL, ((u[r] | u[r + 1] | u[r + 2] | u[r + 3]) >> 16) != 0u)) {
-                    const uint32_t t0 = tpose(__byte_perm(u[r], u[r + 1], 0x5410), tc);
-                    const uint32_t t1 = tpose(__byte_perm(u[r + 2], u[r + 3], 0x5410), tc);
-                    const unsigned m = __ballot_sync(FULL, (t0 | t1) != 0u);
-                    np = 32 - __clz((m & 0xffffu) | (m >> 16));
-                    const unsigned pp = seg + lo + 16 * k + (hmask & 4);
-                    sts_u32_if(pp, t0, k, np);
-                    sts_u32_if(pp + 8, t1, k, np);
-                } else {
-                    const uint32_t t0 = tpose(u[r], tc), t1 = tpose(u[r + 1], tc);
-                    const uint32_t t2 = tpose(u[r + 2], tc), t3 = tpose(u[r + 3], tc);
-                    np = 32 - __clz(__ballot_sync(FULL, (t0 | t1 | t2 | t3) != 0u));
-                    sts_u128_if(seg + lo + 16 * lane, t0, t1, t2, t3, lane, np);
-                }
-                wacc[0] |= (uint32_t)width_byte(np) << (8 * (r / 4));
-                lo += 16 * np;
-            }
-        }
-    }
-    // one store of the group's width bytes (wb is 16-byte aligned per group
-    // at L = 16, 8 at L = 32, 4 at L = 64, 2 at L = 128)
-    if (L == 16) sts_if(wb, make_uint4(wacc[0], wacc[1], wacc[2], wacc[3]), lane == 0);
-    else if (L == 32) sts_if(wb, make_uint2(wacc[0], wacc[1]), lane == 0 && !quad);
-    else if (L == 64) sts_if(wb, wacc[0], lane == 0);
-    else sts_if(wb, (unsigned short)wacc[0], lane == 0);
-    return lo;
+    const uintptr_t a0 = (uintptr_t)p, a1 = a0 + len;
+    const uintptr_t s0 = (a0 + 15) & ~(uintptr_t)15, s1 = a1 & ~(uintptr_t)15;
+    if (s1 > s0)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(s0), "r"((unsigned)(s1 - s0))
+                     : "memory");
 }
 
 // ---- encoder tiles -------------------------------------------------------------
@@ -998,22 +330,25 @@ struct EncShared {
 };
 
 // Encoder warp `warp`'s unit of one tile: quantize, delta-code and bit-plane
-// pack its U rows, through its shared-memory `stage` (SR rows at a time),
-// into its ring segment `seg`, and its width bytes into `wb`; returns the
-// segment's size.  HAS_CIN: decode `it.cin` first (same block size, unit
-// offsets from k_wscan) and add the local chunk; the FP32 sum then goes to
-// `it.raw_out` when that is set.  Null pointers switch a step off.  HEADS
-// (block heads stored apart, single unpacked streams) writes the heads
+// pack its U rows, 32 rows at a time (zc_rows.cuh), into its ring segment
+// `seg`, and its width bytes into `wb`; returns the segment's size.  `bufs`
+// (shared memory) are the warp's two group buffers: the next group's values
+// arrive in one while the other is encoded and its payload, built over the
+// values, copied to the ring.  HAS_CIN: decode `it.cin` first (same block
+// size, unit offsets from k_wscan) and add the local chunk; the FP32 sum then
+// goes to `it.raw_out` when that is set.  Null pointers switch a step off.
+// HEADS (block heads stored apart, single unpacked streams) writes the heads
 // straight to their fixed place in the output.  Thread 0 fills the slot's
 // scalars.
-template <int LOG2L, int U, bool HAS_CIN, typename TX, bool HEADS = false, int SR = 32>
+template <int LOG2L, int U, bool HAS_CIN, typename TX, bool HEADS = false>
 __device__ __forceinline__ int enc_tile(const Launch& P, const Item& it, unsigned item_idx,
                                         unsigned tile_in_item, uint8_t* seg, uint8_t* wb,
-                                        uint8_t* stage, TileSlot& S, EncShared& es)
+                                        unsigned bufs, TileSlot& S, EncShared& es)
 {
     static_assert(!HEADS || !HAS_CIN, "heads apart: compression only");
+    static_assert(U % GROWS == 0, "whole groups");
     constexpr int L = 1 << LOG2L;
-    constexpr int BU = U * 32 / L;  // blocks per warp unit
+    constexpr int BPG = GELEMS / L;  // blocks per group
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     Ctl* ctl = P.ctl;
     const unsigned long long n = it.n;
@@ -1030,6 +365,13 @@ __device__ __forceinline__ int enc_tile(const Launch& P, const Item& it, unsigne
         S.head = first ? 32ull + wbytes + (HEADS ? ceil16(3ull * nb) : 0ull) : 0ull;
         S.pub = do_enc;
     }
+    const int un = ue0 < n ? (int)min(n - ue0, (unsigned long long)(U * 32)) : 0;  // unit elements
+    const TX* const xp = (const TX*)it.x + ue0;
+    const bool vec = ((uintptr_t)xp & 15u) == 0;
+    if (un > 0) {
+        if (lane == 0) prefetch_l2(xp, (unsigned)un * (unsigned)sizeof(TX));
+        stage_in<TX>(xp, min(un, GELEMS), vec, bufs);
+    }
     float two_eb_in = 0.0f;
     if (do_cin) {
         if (tid == 0) {
@@ -1040,178 +382,121 @@ __device__ __forceinline__ int enc_tile(const Launch& P, const Item& it, unsigne
             if (es.hdr_bad) S.pub = 0;
         }
         bar_sync_n(BAR_ENCW, NTHREADS);
-        if (es.hdr_bad) return 0;
+        if (es.hdr_bad) {
+            cp_wait<0>();
+            return 0;
+        }
         two_eb_in = __fadd_rn(es.eb_in, es.eb_in);
     }
-    float eb = it.eb, two_eb = it.two_eb, inv = it.inv;
+    if (un == 0) return 0;
+    EncArgs A;
+    A.eb = it.eb;
+    A.two_eb = it.two_eb;
+    A.inv = it.inv;
     if (P.eb_from_ctl) {
-        eb = ctl->eb;
-        two_eb = ctl->two_eb;
-        inv = ctl->inv;
+        A.eb = ctl->eb;
+        A.two_eb = ctl->two_eb;
+        A.inv = ctl->inv;
     }
-
-    const TpC tc = tp_consts(lane);
+    A.r0 = 0;
+    A.carry = 0u;
+    unsigned long long pos = 0ull;  // received stream: payload position of the group
+    uint32_t wv = 0u;               // and its width byte(s) of this lane's row
+    if (do_cin) {
+        const unsigned slot = S.g * NWARPS + warp;
+        pos = 32ull + wbytes + (dcheck(ctl, slot < P.ws_cap, slot) ? P.offs[slot] : 0ull);
+        wv = load_widths<LOG2L>(it.cin, nb, ue0 >> LOG2L);
+    }
     int err = 0;
-    int lo = 0;
-    // The unit's payload is staged in shared memory (`stage`, this warp's
-    // stage_bytes(SR)), SR rows at a time, and flushed to its ring segment
-    // `seg` with 16-byte copies.  The
-    // stage holds ring bytes [sbase, lo) (sbase 16-byte aligned); a flush
-    // copies them and keeps the partial last 16 bytes at the stage start.
-    static_assert(SR % GR == 0 && U % SR == 0, "stage geometry");
-    __shared__ __align__(16) int2 meta_all[HAS_CIN ? NWARPS : 1][HAS_CIN ? BU : 1];
-    const unsigned stage_s = (unsigned)__cvta_generic_to_shared(stage);
-    int sbase = 0;
-    auto flush = [&](int lo_end) {
-        int n16 = (lo_end - sbase + 15) >> 4;
-        if (!dcheck(ctl, sbase + 16 * n16 <= seg_bytes(U), ue0)) n16 = 0;
-        for (int i = lane; i < n16; i += 32)
-            ((uint4*)(seg + sbase))[i] = ((const uint4*)stage)[i];
-        const int nbase = lo_end & ~15;
-        __syncwarp();
-        if (lane == 0 && nbase != sbase && (lo_end & 15) != 0)
-            ((uint4*)stage)[0] = ((const uint4*)stage)[(nbase - sbase) >> 4];
-        __syncwarp();
-        sbase = nbase;
-    };
-    if (do_enc && it.x != nullptr && ue0 + U * 32 <= n) {
-        // a whole unit (every unit but the last of a stream): no tails, and
-        // few live values, so the group loop stays in registers
-        const TX* const xb = (const TX*)it.x + ue0 + lane;
-        if (lane == 0) {
-            // the whole unit's input into L2 at once (16-byte aligned inner range)
-            const uintptr_t a0 = (uintptr_t)((const TX*)it.x + ue0), a1 = a0 + U * 32 * sizeof(TX);
-            const uintptr_t s0 = (a0 + 15) & ~(uintptr_t)15, s1 = a1 & ~(uintptr_t)15;
-            if (s1 > s0)
-                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(s0),
-                             "r"((unsigned)(s1 - s0))
-                             : "memory");
-        }
-        const uint8_t* src = nullptr;
-        int2* meta = nullptr;
-        bool narrow = false, narrow11 = false;
-        if constexpr (HAS_CIN) {
-            meta = meta_all[warp];
-            if (do_cin)
-                src = it.cin + unit_meta<LOG2L, U>(P, it, S.g * NWARPS + warp, ue0, meta, narrow,
-                                                   narrow11);
-        }
+    int sbase = 0;  // ring bytes written; the payload so far is sbase + A.r0
 #pragma unroll 1
-        for (int gi = 0; gi < U / GR; ++gi) {
-            float acc[GR];
-#pragma unroll
-            for (int r = 0; r < GR; ++r) acc[r] = load_x<TX>(xb, gi * GR * 32 + r * 32);
-            if constexpr (HAS_CIN) {
-                if (do_cin) {
-                    float dv[GR];
-                    if (narrow11) decode_group<LOG2L, true, false, true>(src, meta, gi, two_eb_in, dv, tc);
-                    else if (narrow) decode_group<LOG2L, true>(src, meta, gi, two_eb_in, dv, tc);
-                    else decode_group<LOG2L, false>(src, meta, gi, two_eb_in, dv, tc);
-#pragma unroll
-                    for (int r = 0; r < GR; ++r) acc[r] = __fadd_rn(dv[r], acc[r]);
-                }
-                if (it.raw_out != nullptr) {
-                    float* op = (float*)it.raw_out + ue0 + gi * GR * 32 + lane;
-#pragma unroll
-                    for (int r = 0; r < GR; ++r) op[r * 32] = acc[r];
-                }
-            }
-            const int b0 = L >= 32 ? gi * GR / (L / 32) : gi * GR * 2;
-            uint8_t* hout = nullptr;
-            if (HEADS) hout = it.out + 32 + wbytes + 3ull * ((ue0 >> LOG2L) + b0);
-            if (HEADS && DEBUG_BUILD)
-                dcheck(ctl, 32 + wbytes + 3ull * ((ue0 >> LOG2L) + b0 + GR * 32 / L) <= it.out_cap,
-                       ue0);
-            if (dcheck(ctl, lo - sbase + seg_bytes(GR) <= stage_bytes(SR), ue0))
-                lo = encode_group<LOG2L, true, HEADS>(acc, GR * 32, eb, two_eb, inv, stage_s - sbase,
-                                                      lo, wb + b0, err, tc, hout);
-            if ((gi + 1) % (SR / GR) == 0) flush(lo);
+    for (int g = 0; g * GELEMS < un; ++g) {
+        const int e0 = g * GELEMS;
+        A.nrem = min(un - e0, GELEMS);
+        A.buf = bufs + (g & 1) * GBUF;
+        const bool more = e0 + GELEMS < un;
+        if (more) {
+            stage_in<TX>(xp + e0 + GELEMS, min(un - e0 - GELEMS, GELEMS), vec,
+                         bufs + ((g + 1) & 1) * GBUF);
+            cp_wait<1>();
+        } else {
+            cp_wait<0>();
         }
-    } else if (ue0 < n) {
-        const uint8_t* src = nullptr;
-        int2* meta = nullptr;
-        bool narrow = false, narrow11 = false;
+        __syncwarp();
         if constexpr (HAS_CIN) {
-            meta = meta_all[warp];
-            if (do_cin)
-                src = it.cin + unit_meta<LOG2L, U>(P, it, S.g * NWARPS + warp, ue0, meta, narrow,
-                                                   narrow11);
-        }
-        // the next group's input is loaded while the current one is encoded
-        float xn[GR];
-        const TX* const xbase = it.x != nullptr ? (const TX*)it.x + ue0 + lane : nullptr;
-        {
-            const int nrem0 = (int)min(n - ue0, (unsigned long long)(GR * 32));
-#pragma unroll
-            for (int r = 0; r < GR; ++r)
-                xn[r] = (xbase != nullptr && r * 32 + lane < nrem0) ? load_x<TX>(xbase, r * 32) : 0.0f;
-        }
-#pragma unroll 1
-        for (int gi = 0; gi < U / GR; ++gi) {
-            const unsigned long long e0 = ue0 + (unsigned long long)gi * GR * 32;
-            if (e0 >= n) break;
-            const int nrem = (int)min(n - e0, (unsigned long long)(GR * 32));
-            float acc[GR];
-#pragma unroll
-            for (int r = 0; r < GR; ++r) acc[r] = xn[r];
-            if (gi + 1 < U / GR && e0 + GR * 32 < n) {
-                const TX* xp = xbase + (gi + 1) * GR * 32;
-                if (xbase != nullptr && e0 + 2 * GR * 32 <= n) {
-#pragma unroll
-                    for (int r = 0; r < GR; ++r) xn[r] = load_x<TX>(xp, r * 32);
-                } else {
-                    const int nrem1 = (int)min(n - e0 - GR * 32, (unsigned long long)(GR * 32));
-#pragma unroll
-                    for (int r = 0; r < GR; ++r)
-                        xn[r] = (xbase != nullptr && r * 32 + lane < nrem1) ? load_x<TX>(xp, r * 32)
-                                                                             : 0.0f;
+            if (do_cin) {
+                int np, np2, at;
+                bool bad = false;
+                const int tot = rows_meta<LOG2L>(wv, np, np2, at, bad);
+                if (bad) fail(ctl, ZC_ERR_FORMAT, ue0 + e0);
+                const bool ok = pos + (unsigned long long)tot <= it.cin_cap;
+                if (!ok) {
+                    if (lane == 0) fail(ctl, ZC_ERR_FORMAT, S.g * NWARPS + warp);
+                    np = np2 = 0;
                 }
-            }
-            if constexpr (HAS_CIN) {
-                if (do_cin) {
-                    float dv[GR];
-                    if (narrow11) decode_group<LOG2L, true, false, true>(src, meta, gi, two_eb_in, dv, tc);
-                    else if (narrow) decode_group<LOG2L, true>(src, meta, gi, two_eb_in, dv, tc);
-                    else decode_group<LOG2L, false>(src, meta, gi, two_eb_in, dv, tc);
-#pragma unroll
-                    for (int r = 0; r < GR; ++r) acc[r] = __fadd_rn(dv[r], acc[r]);
+                const PlaneSrc<false> ps{0u, it.cin + pos + at};
+                if (more) wv = load_widths<LOG2L>(it.cin, nb, (ue0 + e0 + GELEMS) >> LOG2L);
+                pos += (unsigned long long)tot;
+                const unsigned row = A.buf + lane * 128 + ((lane & 7) << 4);
+                decode_rows<LOG2L, false, false>(
+                    ps, np, np2, 0, 0, two_eb_in, [] {},
+                    [&](int c, const float v[4]) {
+                        const uint4 x = lds128(row ^ (c << 4));
+                        sts128(row ^ (c << 4), __float_as_uint(__fadd_rn(v[0], __uint_as_float(x.x))),
+                               __float_as_uint(__fadd_rn(v[1], __uint_as_float(x.y))),
+                               __float_as_uint(__fadd_rn(v[2], __uint_as_float(x.z))),
+                               __float_as_uint(__fadd_rn(v[3], __uint_as_float(x.w))));
+                    });
+                __syncwarp();
+                if (A.nrem < GELEMS) {  // the padding repeats the last sum
+                    const uint32_t v = lds32(elem_addr<float>(A.buf, A.nrem - 1));
+                    __syncwarp();
+                    for (int e = A.nrem + lane; e < GELEMS; e += 32) sts32(elem_addr<float>(A.buf, e), v);
+                    __syncwarp();
                 }
-            }
-            if (HAS_CIN && it.raw_out != nullptr) {
-                float* op = (float*)it.raw_out + e0 + lane;
-                const bool check = do_cin && !do_enc;
+                if (!do_enc) {  // the quantizer does not see these sums
+                    float m = 0.0f;
 #pragma unroll
-                for (int r = 0; r < GR; ++r) {
-                    if (r * 32 + lane < nrem) {
-                        op[r * 32] = acc[r];
-                        if (check && !isfinite(acc[r])) err |= ZC_ERR_NONFINITE;
+                    for (int c = 0; c < 8; ++c) {
+                        const uint4 x = lds128(row ^ (c << 4));
+                        m = max3_abs_nan(m, __uint_as_float(x.x), __uint_as_float(x.y));
+                        m = max3_abs_nan(m, __uint_as_float(x.z), __uint_as_float(x.w));
                     }
+                    if (!isfinite(m)) err |= ZC_ERR_NONFINITE;
                 }
             }
-            if (do_enc) {
-                const int b0 = L >= 32 ? gi * GR / (L / 32) : gi * GR * 2;
-                uint8_t* hout = nullptr;
-                if (HEADS) hout = it.out + 32 + wbytes + 3ull * ((ue0 >> LOG2L) + b0);
-                if (!dcheck(ctl, lo - sbase + seg_bytes(GR) <= stage_bytes(SR), e0))
-                    ;
-                else if (nrem == GR * 32)
-                    lo = encode_group<LOG2L, true, HEADS>(acc, nrem, eb, two_eb, inv,
-                                                          stage_s - sbase, lo, wb + b0, err, tc,
-                                                          hout);
-                else
-                    lo = encode_group<LOG2L, false, HEADS>(acc, nrem, eb, two_eb, inv,
-                                                           stage_s - sbase, lo, wb + b0, err, tc,
-                                                           hout);
-                if ((gi + 1) % (SR / GR) == 0) flush(lo);
+            if (it.raw_out != nullptr) {
+                float* const op = (float*)it.raw_out + ue0 + e0;
+                stage_out<float>(op, A.nrem, ((uintptr_t)op & 15u) == 0, A.buf);
             }
         }
-        if (do_enc) flush(lo);
+        if (do_enc) {
+            const unsigned long long bg = (ue0 + e0) >> LOG2L;  // first block of the group
+            if (HEADS) {
+                A.hout = it.out + 32 + wbytes + 3ull * bg;
+                if (DEBUG_BUILD)
+                    dcheck(ctl, 32 + wbytes + 3ull * min(bg + BPG, nb) <= it.out_cap, ue0);
+            }
+            A.wb = (unsigned)__cvta_generic_to_shared(wb) + g * BPG;
+            const int end = A.r0 + encode_rows<LOG2L, TX, HEADS>(A, err);
+            __syncwarp();
+            // the payload to the ring, in 16-byte chunks; the partial last
+            // one is written now and again, complete, with the next group
+            int n16 = (end + 15) >> 4;
+            if (!dcheck(ctl, end <= GBUF && sbase + 16 * n16 <= seg_bytes(U), ue0)) n16 = 0;
+            for (int i = lane; i < n16; i += 32)
+                ((uint4*)(seg + sbase))[i] = lds128(A.buf + 16 * i);
+            if (lane < 4) A.carry = lds32(A.buf + (end & ~15) + 4 * lane);
+            sbase += end & ~15;
+            A.r0 = end & 15;
+        }
+        __syncwarp();  // the buffer is free
     }
     {
         const unsigned bad = __ballot_sync(FULL, err != 0);
         if (bad && lane == __ffs(bad) - 1) fail(ctl, (unsigned)err, ue0);
     }
-    return do_enc ? lo : 0;
+    return do_enc ? sbase + A.r0 : 0;
 }
 
 // Stores of one encoded tile once its place is known: every encoder warp
@@ -1483,15 +768,14 @@ __device__ __forceinline__ void resolve_slot(const Launch& P, TileSlot& S, unsig
 // BAR_RES + s, where the encoder warps wait NS - 1 tiles later before
 // storing it.  A slot's barriers are used again only after both sides have
 // passed them, and every path through the loops meets every barrier.
-template <int U, bool SINGLE, typename Src, typename Enc, typename Fin>
+template <int U, typename Src, typename Enc, typename Fin>
 __device__ __forceinline__ void enc_pipeline(const Launch& P, const Src& src, Enc enc, Fin fin)
 {
     constexpr int NS = enc_slots(U);  // tiles in flight
     constexpr int D = NS - 1;         // tiles between a tile's encoding and its stores
     __shared__ TileSlot slots[NS];
     __shared__ EncShared es;
-    extern __shared__ __align__(16) uint8_t dsm[];  // width bytes [slot][warp][2U] (, stages)
-    __shared__ __align__(16) uint8_t stage_static[SINGLE ? 1 : NWARPS][SINGLE ? 16 : stage_bytes(32)];
+    extern __shared__ __align__(128) uint8_t dsm[];  // group buffers, width bytes [slot][warp][2U]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // a relative bound comes from the range kernel launched just before, the
     // fused ring step's offsets and tile map from the kernels before it: an
@@ -1519,11 +803,8 @@ __device__ __forceinline__ void enc_pipeline(const Launch& P, const Src& src, En
     uint8_t* const ring = P.ring + (unsigned long long)blockIdx.x * ring_cta_bytes(U);
     if (warp < NWARPS) {
         auto seg_of = [&](int s) { return ring + (unsigned long long)(s * NWARPS + warp) * seg_bytes(U); };
-        auto wb_of = [&](int s) { return dsm + (s * NWARPS + warp) * (U * 2); };
-        auto stage_of = [&]() -> uint8_t* {
-            if constexpr (SINGLE) return dsm + enc_wb_bytes(U) + warp * stage_bytes(stage_rows(U, true));
-            else return stage_static[warp];
-        };
+        auto wb_of = [&](int s) { return dsm + NWARPS * 2 * GBUF + (s * NWARPS + warp) * (U * 2); };
+        const unsigned bufs = (unsigned)__cvta_generic_to_shared(dsm) + warp * (2 * GBUF);
         auto store = [&](int q) {
             bar_sync_n(BAR_RES + q, ENC_THREADS);
             const TileSlot& Q = slots[q];
@@ -1552,7 +833,7 @@ __device__ __forceinline__ void enc_pipeline(const Launch& P, const Src& src, En
                 const Item it = src.get(S.item);
                 const unsigned t = S.g - it.tile_begin;
                 if (tid == 0) S.tile = t;
-                lo = enc(it, S.item, t, seg_of(s), wb_of(s), stage_of(), S, es);
+                lo = enc(it, S.item, t, seg_of(s), wb_of(s), bufs, S, es);
             }
             if (lane == 0) {
                 S.segsz[warp] = lo;
@@ -1596,12 +877,11 @@ __device__ __forceinline__ void enc_pipeline(const Launch& P, const Src& src, En
 template <int LOG2L, int U, typename TX, bool HEADS = false>
 __global__ void __launch_bounds__(ENC_THREADS, ENC_CTAS_PER_SM) k_compress(const Launch P)
 {
-    enc_pipeline<U, true>(
+    enc_pipeline<U>(
         P, ItemsSrc{P},
-        [&](const Item& it, unsigned idx, unsigned t, uint8_t* seg, uint8_t* wb, uint8_t* stage,
+        [&](const Item& it, unsigned idx, unsigned t, uint8_t* seg, uint8_t* wb, unsigned bufs,
             TileSlot& S, EncShared& es) {
-            return enc_tile<LOG2L, U, false, TX, HEADS, stage_rows(U, true)>(P, it, idx, t, seg, wb,
-                                                                          stage, S, es);
+            return enc_tile<LOG2L, U, false, TX, HEADS>(P, it, idx, t, seg, wb, bufs, S, es);
         },
         [&](const Item& it, unsigned idx, unsigned t, unsigned g, const TileSlot& S,
             const uint8_t* seg, const uint8_t* wb) { fin_tile<LOG2L, U, false, HEADS>(P, it, idx, t, g, S, seg, wb); });
@@ -1611,12 +891,11 @@ template <int LOG2L, int U, typename TX>
 __global__ void __launch_bounds__(ENC_THREADS, ENC_CTAS_PER_SM) k_scatter(const Launch P,
                                                                           const ScatterParams SP)
 {
-    enc_pipeline<U, true>(
+    enc_pipeline<U>(
         P, ScatterSrc{P, SP},
-        [&](const Item& it, unsigned idx, unsigned t, uint8_t* seg, uint8_t* wb, uint8_t* stage,
+        [&](const Item& it, unsigned idx, unsigned t, uint8_t* seg, uint8_t* wb, unsigned bufs,
             TileSlot& S, EncShared& es) {
-            return enc_tile<LOG2L, U, false, TX, false, stage_rows(U, true)>(P, it, idx, t, seg, wb,
-                                                                          stage, S, es);
+            return enc_tile<LOG2L, U, false, TX>(P, it, idx, t, seg, wb, bufs, S, es);
         },
         [&](const Item& it, unsigned idx, unsigned t, unsigned g, const TileSlot& S,
             const uint8_t* seg, const uint8_t* wb) { fin_tile<LOG2L, U, false>(P, it, idx, t, g, S, seg, wb); });
@@ -1625,11 +904,11 @@ __global__ void __launch_bounds__(ENC_THREADS, ENC_CTAS_PER_SM) k_scatter(const 
 template <int LOG2L, int U>
 __global__ void __launch_bounds__(ENC_THREADS, ENC_CTAS_PER_SM) k_reduce(const Launch P)
 {
-    enc_pipeline<U, false>(
+    enc_pipeline<U>(
         P, ItemsSrc{P},
-        [&](const Item& it, unsigned idx, unsigned t, uint8_t* seg, uint8_t* wb, uint8_t* stage,
+        [&](const Item& it, unsigned idx, unsigned t, uint8_t* seg, uint8_t* wb, unsigned bufs,
             TileSlot& S, EncShared& es) {
-            return enc_tile<LOG2L, U, true, float>(P, it, idx, t, seg, wb, stage, S, es);
+            return enc_tile<LOG2L, U, true, float>(P, it, idx, t, seg, wb, bufs, S, es);
         },
         [&](const Item& it, unsigned idx, unsigned t, unsigned g, const TileSlot& S,
             const uint8_t* seg, const uint8_t* wb) { fin_tile<LOG2L, U, true>(P, it, idx, t, g, S, seg, wb); });
@@ -1643,24 +922,24 @@ __global__ void __launch_bounds__(ENC_THREADS, ENC_CTAS_PER_SM) k_reduce(const L
 template <int U>
 __global__ void __launch_bounds__(ENC_THREADS, ENC_CTAS_PER_SM) k_batch(const Launch P)
 {
-    enc_pipeline<U, false>(
+    enc_pipeline<U>(
         P, ItemsSrc{P},
-        [&](const Item& it, unsigned idx, unsigned t, uint8_t* seg, uint8_t* wb, uint8_t* stage,
+        [&](const Item& it, unsigned idx, unsigned t, uint8_t* seg, uint8_t* wb, unsigned bufs,
             TileSlot& S, EncShared& es) -> int {
             const bool f32 = it.x_dtype == ZC_F32;
             switch (it.log2L) {
             case 4:
-                return f32 ? enc_tile<4, U, false, float>(P, it, idx, t, seg, wb, stage, S, es)
-                           : enc_tile<4, U, false, uint16_t>(P, it, idx, t, seg, wb, stage, S, es);
+                return f32 ? enc_tile<4, U, false, float>(P, it, idx, t, seg, wb, bufs, S, es)
+                           : enc_tile<4, U, false, uint16_t>(P, it, idx, t, seg, wb, bufs, S, es);
             case 5:
-                return f32 ? enc_tile<5, U, false, float>(P, it, idx, t, seg, wb, stage, S, es)
-                           : enc_tile<5, U, false, uint16_t>(P, it, idx, t, seg, wb, stage, S, es);
+                return f32 ? enc_tile<5, U, false, float>(P, it, idx, t, seg, wb, bufs, S, es)
+                           : enc_tile<5, U, false, uint16_t>(P, it, idx, t, seg, wb, bufs, S, es);
             case 6:
-                return f32 ? enc_tile<6, U, false, float>(P, it, idx, t, seg, wb, stage, S, es)
-                           : enc_tile<6, U, false, uint16_t>(P, it, idx, t, seg, wb, stage, S, es);
+                return f32 ? enc_tile<6, U, false, float>(P, it, idx, t, seg, wb, bufs, S, es)
+                           : enc_tile<6, U, false, uint16_t>(P, it, idx, t, seg, wb, bufs, S, es);
             case 7:
-                return f32 ? enc_tile<7, U, false, float>(P, it, idx, t, seg, wb, stage, S, es)
-                           : enc_tile<7, U, false, uint16_t>(P, it, idx, t, seg, wb, stage, S, es);
+                return f32 ? enc_tile<7, U, false, float>(P, it, idx, t, seg, wb, bufs, S, es)
+                           : enc_tile<7, U, false, uint16_t>(P, it, idx, t, seg, wb, bufs, S, es);
             default: return enc_raw<U>(it, t, S);
             }
         },
@@ -1969,48 +1248,92 @@ __device__ __forceinline__ void unit_raw_copy(const Item& it, int src_dtype, uns
     }
 }
 
+// One warp unit of a coded stream (zc_rows.cuh), 32 rows at a time.  `bufs`:
+// the warp's two group buffers; a group's payload arrives in its buffer (both
+// groups' copies are in flight before the first is decoded), and the decoded
+// rows take its place before they are stored, 16 bytes a lane.
+// off_local >= 0: the unit's payload offset found by the caller (a small
+// item's decoder CTA), in place of the width scan's P.offs[slot].
 template <int LOG2L, typename TO, bool HEADS = false>
 __device__ __forceinline__ void unit_decode(const Launch& P, const Item& it, unsigned slot,
-                                            unsigned long long ue0, float two_eb, int2* meta,
+                                            unsigned long long ue0, float two_eb, unsigned bufs,
                                             long long off_local)
 {
+    static_assert(DEC_U == 2 * GROWS, "two groups per unit");
+    constexpr int L = 1 << LOG2L;
+    constexpr int RPB = Blk<LOG2L>::RPB;
     const int lane = threadIdx.x & 31;
-    const TpC tc = tp_consts(lane);
-    bool narrow;
-    bool narrow11;
-    const uint8_t* src = it.cin + unit_meta<LOG2L, DEC_U, HEADS>(P, it, slot, ue0, meta, narrow,
-                                                                 narrow11, off_local);
-    const uint8_t* hsrc = nullptr;  // heads apart: the heads of this unit's blocks
-    if (HEADS) {
-        const unsigned long long nb = (it.n + (1ull << LOG2L) - 1) >> LOG2L;
-        hsrc = it.cin + 32 + ceil16(nb) + 3ull * (ue0 >> LOG2L);
-    }
-#pragma unroll 1
-    for (int gi = 0; gi < DEC_U / GR; ++gi) {
-        const unsigned long long e0 = ue0 + (unsigned long long)gi * GR * 32;
-        if (e0 >= it.n) break;
-        const int nrem = (int)min(it.n - e0, (unsigned long long)(GR * 32));
-        float acc[GR];
-        if (!HEADS && narrow11) decode_group<LOG2L, true, false, true>(src, meta, gi, two_eb, acc, tc);
-        else if (narrow) decode_group<LOG2L, true, HEADS>(src, meta, gi, two_eb, acc, tc, hsrc);
-        else decode_group<LOG2L, false, HEADS>(src, meta, gi, two_eb, acc, tc, hsrc);
-        TO* op = (TO*)it.raw_out + e0 + lane;
-        if (nrem == GR * 32) {
-#pragma unroll
-            for (int r = 0; r < GR; ++r) {
-                if (sizeof(TO) == 4) ((float*)op)[r * 32] = acc[r];
-                else ((uint16_t*)op)[r * 32] = f32_to_bf16(acc[r]);
-            }
+    const unsigned long long nb = (it.n + L - 1) >> LOG2L;
+    const unsigned long long b0 = ue0 >> LOG2L;
+    const int un = (int)min(it.n - ue0, (unsigned long long)(DEC_U * 32));
+    const uint32_t wv1 = load_widths<LOG2L>(it.cin, nb, b0 + GELEMS / L);
+    const uint32_t wv0 = load_widths<LOG2L>(it.cin, nb, b0);
+    const bool slot_ok = off_local >= 0 || dcheck(P.ctl, slot < P.ws_cap, slot);
+    unsigned long long pos = 32ull + ceil16(nb) + (HEADS ? ceil16(3ull * nb) : 0ull) +
+                             (off_local >= 0 ? (unsigned long long)off_local
+                                             : (slot_ok ? P.offs[slot] : 0ull));
+    struct Group {
+        int np, np2;
+        unsigned sp;  // the lane's first plane word in the group buffer
+    };
+    // Requests the payload of a group (at `pos`) into its buffer.  The 16-byte
+    // chunks it touches lie inside the stream (16-byte aligned and padded).
+    auto fetch = [&](uint32_t wv, unsigned buf) {
+        Group G;
+        int at;
+        bool bad = false;
+        const int tot = rows_meta<LOG2L>(wv, G.np, G.np2, at, bad);
+        if (bad) fail(P.ctl, ZC_ERR_FORMAT, b0);
+        const unsigned long long c0 = pos & ~15ull, c1 = ceil16(pos + (unsigned long long)tot);
+        if (slot_ok && c1 <= it.cin_cap) {
+            const uint8_t* const src = it.cin + c0;
+            const int n16 = (int)((c1 - c0) >> 4);
+            for (int i = lane; i < n16; i += 32) cp_async16(buf + 16 * i, src + 16 * i);
         } else {
-#pragma unroll
-            for (int r = 0; r < GR; ++r) {
-                if (r * 32 + lane < nrem) {
-                    if (sizeof(TO) == 4) ((float*)op)[r * 32] = acc[r];
-                    else ((uint16_t*)op)[r * 32] = f32_to_bf16(acc[r]);
-                }
-            }
+            if (lane == 0) fail(P.ctl, ZC_ERR_FORMAT, slot);
+            G.np = G.np2 = 0;
         }
+        cp_commit();
+        G.sp = buf + (unsigned)(pos & 15ull) + at;
+        pos += (unsigned long long)tot;
+        return G;
+    };
+    Group G = fetch(wv0, bufs), G1 = fetch(wv1, bufs + GBUF);
+#pragma unroll 1
+    for (int g = 0; g * GELEMS < un; ++g) {
+        const int nrem = min(un - g * GELEMS, GELEMS);
+        const unsigned buf = bufs + g * GBUF;
+        int h0 = 0, h16 = 0;
+        if (HEADS) {  // the heads of this lane's blocks
+            const unsigned long long b = b0 + (unsigned)(g * (GELEMS / L)) +
+                                         (L == 16 ? 2 * lane : lane / RPB);
+            const uint8_t* const hp = it.cin + 32 + ceil16(nb) + 3ull * b;
+            if ((lane & (RPB - 1)) == 0 && b < nb) h0 = load_head(hp);
+            if (L == 16 && b + 1 < nb) h16 = load_head(hp + 3);
+        }
+        if (g == 0) cp_wait<1>();
+        else cp_wait<0>();
+        __syncwarp();
+        const PlaneSrc<true> ps{G.sp, nullptr};
+        const unsigned row = sizeof(TO) == 4 ? buf + lane * 128 + ((lane & 7) << 4)
+                                             : buf + lane * 64 + (((lane >> 1) & 3) << 4);
+        decode_rows<LOG2L, true, HEADS>(
+            ps, G.np, G.np2, h0, h16, two_eb, [] { __syncwarp(); },
+            [&](int c, const float v[4]) {
+                if (sizeof(TO) == 4) {
+                    sts128(row ^ (c << 4), __float_as_uint(v[0]), __float_as_uint(v[1]),
+                           __float_as_uint(v[2]), __float_as_uint(v[3]));
+                } else {
+                    sts64((row ^ ((c >> 1) << 4)) + (c & 1) * 8, f32_to_bf16x2(v[0], v[1]),
+                          f32_to_bf16x2(v[2], v[3]));
+                }
+            });
+        __syncwarp();
+        TO* const op = (TO*)it.raw_out + ue0 + g * GELEMS;
+        stage_out<TO>(op, nrem, ((uintptr_t)op & 15u) == 0, buf);
+        G = G1;
     }
+    cp_wait<0>();
 }
 
 // Items of at most DEC_LOCAL_TILES decode tiles (planned with no width-scan
@@ -2074,7 +1397,7 @@ __device__ __forceinline__ unsigned long long local_unit_offset(const Item& it, 
 template <bool BATCH>
 __device__ __forceinline__ void decompress_tile(const Launch& P)
 {
-    __shared__ __align__(16) int2 meta[NWARPS][DEC_U * 2];
+    extern __shared__ __align__(128) uint8_t dsm[];
     const unsigned tile = blockIdx.x;
     unsigned idx = 0;
     if (P.tile_map != nullptr) {
@@ -2094,6 +1417,7 @@ __device__ __forceinline__ void decompress_tile(const Launch& P)
     const int warp = threadIdx.x >> 5;
     const unsigned long long ue0 = ((unsigned long long)t * NWARPS + warp) * (DEC_U * 32);
     const unsigned slot = tile * NWARPS + warp;
+    const unsigned bufs = (unsigned)__cvta_generic_to_shared(dsm) + warp * (2 * GBUF);
     float eb_in;
     const int lg = check_header(it, P.ctl, idx, -1, eb_in, threadIdx.x == 0 && t == 0);
     long long loff = -1;  // the unit's payload offset, when this CTA finds it
@@ -2109,26 +1433,26 @@ __device__ __forceinline__ void decompress_tile(const Launch& P)
     const float two = __fadd_rn(eb_in, eb_in);
     if (it.out_dtype == ZC_F32) {
         switch (lg) {
-        case 4: unit_decode<4, float>(P, it, slot, ue0, two, meta[warp], loff); return;
-        case 5: unit_decode<5, float>(P, it, slot, ue0, two, meta[warp], loff); return;
-        case 6: unit_decode<6, float>(P, it, slot, ue0, two, meta[warp], loff); return;
-        case 7: unit_decode<7, float>(P, it, slot, ue0, two, meta[warp], loff); return;
-        case 12: unit_decode<4, float, true>(P, it, slot, ue0, two, meta[warp], loff); return;
-        case 13: unit_decode<5, float, true>(P, it, slot, ue0, two, meta[warp], loff); return;
-        case 14: unit_decode<6, float, true>(P, it, slot, ue0, two, meta[warp], loff); return;
-        case 15: unit_decode<7, float, true>(P, it, slot, ue0, two, meta[warp], loff); return;
+        case 4: unit_decode<4, float>(P, it, slot, ue0, two, bufs, loff); return;
+        case 5: unit_decode<5, float>(P, it, slot, ue0, two, bufs, loff); return;
+        case 6: unit_decode<6, float>(P, it, slot, ue0, two, bufs, loff); return;
+        case 7: unit_decode<7, float>(P, it, slot, ue0, two, bufs, loff); return;
+        case 12: unit_decode<4, float, true>(P, it, slot, ue0, two, bufs, loff); return;
+        case 13: unit_decode<5, float, true>(P, it, slot, ue0, two, bufs, loff); return;
+        case 14: unit_decode<6, float, true>(P, it, slot, ue0, two, bufs, loff); return;
+        case 15: unit_decode<7, float, true>(P, it, slot, ue0, two, bufs, loff); return;
         default: break;
         }
     } else {
         switch (lg) {
-        case 4: unit_decode<4, uint16_t>(P, it, slot, ue0, two, meta[warp], loff); return;
-        case 5: unit_decode<5, uint16_t>(P, it, slot, ue0, two, meta[warp], loff); return;
-        case 6: unit_decode<6, uint16_t>(P, it, slot, ue0, two, meta[warp], loff); return;
-        case 7: unit_decode<7, uint16_t>(P, it, slot, ue0, two, meta[warp], loff); return;
-        case 12: unit_decode<4, uint16_t, true>(P, it, slot, ue0, two, meta[warp], loff); return;
-        case 13: unit_decode<5, uint16_t, true>(P, it, slot, ue0, two, meta[warp], loff); return;
-        case 14: unit_decode<6, uint16_t, true>(P, it, slot, ue0, two, meta[warp], loff); return;
-        case 15: unit_decode<7, uint16_t, true>(P, it, slot, ue0, two, meta[warp], loff); return;
+        case 4: unit_decode<4, uint16_t>(P, it, slot, ue0, two, bufs, loff); return;
+        case 5: unit_decode<5, uint16_t>(P, it, slot, ue0, two, bufs, loff); return;
+        case 6: unit_decode<6, uint16_t>(P, it, slot, ue0, two, bufs, loff); return;
+        case 7: unit_decode<7, uint16_t>(P, it, slot, ue0, two, bufs, loff); return;
+        case 12: unit_decode<4, uint16_t, true>(P, it, slot, ue0, two, bufs, loff); return;
+        case 13: unit_decode<5, uint16_t, true>(P, it, slot, ue0, two, bufs, loff); return;
+        case 14: unit_decode<6, uint16_t, true>(P, it, slot, ue0, two, bufs, loff); return;
+        case 15: unit_decode<7, uint16_t, true>(P, it, slot, ue0, two, bufs, loff); return;
         default: break;
         }
     }
@@ -2137,7 +1461,7 @@ __device__ __forceinline__ void decompress_tile(const Launch& P)
 }
 
 template <bool BATCH>
-__global__ void __launch_bounds__(NTHREADS, 5) k_decompress(const Launch P)
+__global__ void __launch_bounds__(NTHREADS, DEC_CTAS_PER_SM) k_decompress(const Launch P)
 {
     decompress_tile<BATCH>(P);
 }

@@ -114,47 +114,6 @@ __device__ __forceinline__ unsigned long long ceil16(unsigned long long v)
     return (v + 15ull) & ~15ull;
 }
 
-// ---- warp bit-matrix transpose -----------------------------------------
-// Lane i holds word u_i; afterwards lane k holds the word whose bit i is bit k
-// of u_i.  Five butterfly stages exchange the off-diagonal sub-blocks of the
-// current block size through one shuffle each: the two byte-granular stages
-// (16- and 8-bit blocks) merge with one byte permute, the three sub-byte
-// stages with one funnel rotate and one bit-select.  The per-lane selectors,
-// rotate counts and masks are computed once per kernel (TpC).  The transpose
-// is its own inverse.  If every u_i < 2^16, packing two rows as
-// u_a | u_b << 16 transposes both at once: lanes 0..15 get the planes of a,
-// lanes 16..31 those of b.
-struct TpC {
-    uint32_t s16, s8, r4, r2, r1, k4, k2, k1;
-};
-__device__ __forceinline__ TpC tp_consts(int lane)
-{
-    TpC c;
-    c.s16 = (lane & 16) ? 0x3276u : 0x5410u;
-    c.s8 = (lane & 8) ? 0x3715u : 0x6240u;
-    c.r4 = (lane & 4) ? 28u : 4u;
-    c.k4 = (lane & 4) ? 0xf0f0f0f0u : 0x0f0f0f0fu;
-    c.r2 = (lane & 2) ? 30u : 2u;
-    c.k2 = (lane & 2) ? 0xccccccccu : 0x33333333u;
-    c.r1 = (lane & 1) ? 31u : 1u;
-    c.k1 = (lane & 1) ? 0xaaaaaaaau : 0x55555555u;
-    return c;
-}
-__device__ __forceinline__ uint32_t tpose(uint32_t u, const TpC& c)
-{
-    uint32_t p = __shfl_xor_sync(FULL, u, 16);
-    u = __byte_perm(u, p, c.s16);
-    p = __shfl_xor_sync(FULL, u, 8);
-    u = __byte_perm(u, p, c.s8);
-    p = __shfl_xor_sync(FULL, u, 4);
-    u = (u & c.k4) | (__funnelshift_l(p, p, c.r4) & ~c.k4);
-    p = __shfl_xor_sync(FULL, u, 2);
-    u = (u & c.k2) | (__funnelshift_l(p, p, c.r2) & ~c.k2);
-    p = __shfl_xor_sync(FULL, u, 1);
-    u = (u & c.k1) | (__funnelshift_l(p, p, c.r1) & ~c.k1);
-    return u;
-}
-
 // Programmatic dependent launch: a kernel launched with programmatic stream
 // serialisation may start while the kernel before it on the stream still
 // runs; grid_dep_wait() blocks until that kernel has completed and its memory
@@ -529,6 +488,14 @@ __device__ __forceinline__ uint16_t f32_to_bf16(float f)
     if ((u & 0x7f800000u) == 0x7f800000u) return (uint16_t)((u >> 16) | ((u & 0x7fffffu) ? 0x40u : 0u));
     u += 0x7fffu + ((u >> 16) & 1u);
     return (uint16_t)(u >> 16);
+}
+
+// Two values as BF16 (round to nearest even), the first in the low half.
+__device__ __forceinline__ uint32_t f32_to_bf16x2(float lo, float hi)
+{
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
 }
 
 }  // namespace zc

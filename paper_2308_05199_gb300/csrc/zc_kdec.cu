@@ -39,12 +39,15 @@ cudaError_t launch_group(Item* items, unsigned n_items, unsigned* part, unsigned
 
 cudaError_t launch_decompress(const Launch& P, unsigned grid, cudaStream_t s, bool after_wscan)
 {
+    const cudaError_t e1 = smem_limit<k_decompress<true>>(DEC_SMEM_BYTES);
+    const cudaError_t e0 = smem_limit<k_decompress<false>>(DEC_SMEM_BYTES);
+    if (e1 != cudaSuccess || e0 != cudaSuccess) return e1 != cudaSuccess ? e1 : e0;
     if (P.items != nullptr) {
-        k_decompress<true><<<grid, NTHREADS, 0, s>>>(P);
+        k_decompress<true><<<grid, NTHREADS, DEC_SMEM_BYTES, s>>>(P);
         return cudaGetLastError();
     }
     if (!after_wscan) {
-        k_decompress<false><<<grid, NTHREADS, 0, s>>>(P);
+        k_decompress<false><<<grid, NTHREADS, DEC_SMEM_BYTES, s>>>(P);
         return cudaGetLastError();
     }
     // launched dependent on the width scan just before it on the stream: its
@@ -52,7 +55,7 @@ cudaError_t launch_decompress(const Launch& P, unsigned grid, cudaStream_t s, bo
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(NTHREADS);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = DEC_SMEM_BYTES;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -52,13 +52,13 @@ cudaError_t launch_compress_lg(int chunks, int x_dtype, const Launch& P, unsigne
     switch (chunks) {
     case 4:
         return launch_typed<k_compress<LG, 32, float>, k_compress<LG, 32, uint16_t>>(
-            x_dtype, enc_smem_bytes(32, true), grid, s, P);
+            x_dtype, enc_smem_bytes(32), grid, s, P);
     case 8:
         return launch_typed<k_compress<LG, 64, float>, k_compress<LG, 64, uint16_t>>(
-            x_dtype, enc_smem_bytes(64, true), grid, s, P);
+            x_dtype, enc_smem_bytes(64), grid, s, P);
     case 16:
         return launch_typed<k_compress<LG, 128, float>, k_compress<LG, 128, uint16_t>>(
-            x_dtype, enc_smem_bytes(128, true), grid, s, P);
+            x_dtype, enc_smem_bytes(128), grid, s, P);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -68,14 +68,14 @@ template <int LG>
 cudaError_t launch_compress_heads_lg(int x_dtype, const Launch& P, unsigned grid, cudaStream_t s)
 {
     return launch_typed<k_compress<LG, 64, float, true>, k_compress<LG, 64, uint16_t, true>>(
-        x_dtype, enc_smem_bytes(64, true), grid, s, P);
+        x_dtype, enc_smem_bytes(64), grid, s, P);
 }
 
 template <int LG, int U>
 static cudaError_t scatter_u(int x_dtype, const Launch& P, const ScatterParams& SP, unsigned grid,
                              cudaStream_t s)
 {
-    const int smem = enc_smem_bytes(U, true);
+    const int smem = enc_smem_bytes(U);
     const cudaError_t e32 = smem_limit<k_scatter<LG, U, float>>(smem);
     const cudaError_t e16 = smem_limit<k_scatter<LG, U, uint16_t>>(smem);
     if (e32 != cudaSuccess || e16 != cudaSuccess) return e32 != cudaSuccess ? e32 : e16;
