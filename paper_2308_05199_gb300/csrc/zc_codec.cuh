@@ -1,31 +1,23 @@
 // zc_codec.cuh -- the tile kernels: compress, decompress, the fused ring step
 // (decompress -> add -> recompress) and the scatter pack.
 //
-// Geometry.  A CTA is 8 warps.  A sub-tile is 2048 consecutive elements: each
-// warp owns R = 8 rows of 32, lane i holding element i of a row.  A block of
-// L elements is L/32 rows (L >= 32) or half a row (L = 16); blocks never
-// straddle warps.
+// Geometry.  A warp unit is U rows of 32 elements (U = 32, 64 or 128), worked
+// on 32 rows at a time, one row per lane (zc_rows.cuh); an encoder tile is 8
+// consecutive units, one per encoder warp of a CTA, a decode tile 8 units of
+// DEC_U rows.  Blocks never straddle groups of 32 rows.
 //
-// Encoding a row: exact quantization, Lorenzo delta against the previous
-// element of the block (the block head against 0), the magnitude shifted left
-// with the sign in bit 0, then one warp bit-matrix transpose: lane k then
-// holds bit plane k-1 (lane 0: the sign plane) of the row, so a block with
-// w-bit deltas is exactly lanes 0 .. w of its rows.  Decoding runs the same
-// steps backwards with an inclusive warp scan in place of the delta.
-//
-// Encoder offsets.  An encoder tile is S sub-tiles.  Every warp appends its
-// blocks' planes to its own shared-memory segment of each sub-tile (the
-// running offset is warp-uniform: no scan), so nothing waits until the whole
-// tile is encoded.  Then one CTA scan over the 8 S segment sizes, one
-// CTA-wide decoupled look-back for the tile's position in the stream, and a
-// coalesced copy of every segment to its place.  The first tile of a stream
+// Encoder offsets.  Every encoder warp appends its blocks' planes to its own
+// ring segment (the running offset is warp-uniform: no scan), so nothing waits
+// until the whole tile is encoded.  The tile's position in the stream comes
+// from a decoupled look-back over the tiles' sizes, run by a resolver warp;
+// then every warp copies its segment to its place.  The first tile of a stream
 // also counts the 32-byte header and the padded width bytes; the last one
 // rounds the stream up to 16 bytes; in packed mode (the scatter pack) one
 // chain runs through all streams.
 //
 // Decoder offsets.  k_wscan reads only the width bytes of a stream and
-// writes the payload offset of every 2048-element decode tile (a chain over
-// 256-tile chunks); decoding then needs no look-back and no barrier.
+// writes the payload offset of every warp unit (a chain over chunks of WSCAN
+// units); decoding then needs no look-back and no barrier.
 #pragma once
 
 #include <type_traits>
@@ -223,16 +215,6 @@ __device__ __forceinline__ uint32_t load_widths(const uint8_t* cin, unsigned lon
                       : (uint32_t)__ldg(cin + 32 + b);
 }
 
-// Requests [p, p + len) into L2 (one bulk prefetch of the 16-byte aligned inner range).
-__device__ __forceinline__ void prefetch_l2(const void* p, unsigned len)
-{
-    const uintptr_t a0 = (uintptr_t)p, a1 = a0 + len;
-    const uintptr_t s0 = (a0 + 15) & ~(uintptr_t)15, s1 = a1 & ~(uintptr_t)15;
-    if (s1 > s0)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(s0), "r"((unsigned)(s1 - s0))
-                     : "memory");
-}
-
 // ---- encoder tiles -------------------------------------------------------------
 // An encoder CTA runs two kinds of warps.  Its NWARPS encoder warps take tiles
 // in ticket order and encode each of the tile's warp units into the CTA's ring
@@ -245,34 +227,55 @@ __device__ __forceinline__ void prefetch_l2(const void* p, unsigned len)
 // overlaps the encoding of the tiles after it.
 
 // Copies `len` bytes (a multiple of UNIT) from the ring (16-byte aligned) to
-// `dst` (UNIT-aligned) with one warp; four loads per lane are in flight.  The
-// staged bytes are dead afterwards: their L2 lines (the segment owns whole
-// 128-byte lines) are dropped without a write-back, so the ring costs no DRAM
-// traffic as long as a tile's lines stay in L2 until it is stored.
+// `dst` (UNIT-aligned) with one warp, through `buf`, a free group buffer of
+// the warp: asynchronous copies bring the bytes into shared memory displaced
+// by dst's distance from a 16-byte boundary (to the word; the odd half word of
+// 2-byte units is shifted on the way out), all of them in flight at once, and
+// 16-byte stores take them out.  (Copied through registers, four 4-byte loads
+// at a time, a 4 KiB segment took eight round trips to L2.)  The staged bytes
+// are dead afterwards: their L2 lines (the segment owns whole 128-byte lines)
+// are dropped without a write-back, so the ring costs no DRAM traffic as long
+// as a tile's lines stay in L2 until it is stored.
 template <int UNIT>
-__device__ __forceinline__ void ring_copy(uint8_t* dst, const uint8_t* src, int len)
+__device__ __forceinline__ void ring_copy(uint8_t* dst, const uint8_t* src, int len, unsigned buf)
 {
+    constexpr int W = UNIT == 2 ? 4 : UNIT;  // bytes per asynchronous copy
+    constexpr int PIECE = GBUF - 32;         // bytes per round (a multiple of 16), with room to displace
     const int lane = threadIdx.x & 31;
-    using T = typename std::conditional<
-        UNIT == 16, uint4,
-        typename std::conditional<UNIT == 8, uint2,
-                                  typename std::conditional<UNIT == 4, unsigned,
-                                                            unsigned short>::type>::type>::type;
-    const int cnt = len / UNIT;
-    for (int b = 0; b < cnt; b += 32 * 4) {
-        T v[4];
+    for (int p = 0; p < len; p += PIECE) {
+        const int n = min(len - p, PIECE);
+        uint8_t* const d = dst + p;
+        const int sh = (int)((uintptr_t)d & 15);
+        const uint8_t* s = src + p + W * lane;
+        unsigned a = buf + (sh & ~(W - 1)) + W * lane;
+#pragma unroll 8
+        for (int o = W * lane; o < n; o += 32 * W, s += 32 * W, a += 32 * W) cp_async_ca<W>(a, s);
+        cp_commit();
+        cp_wait<0>();
+        __syncwarp();
+        uint8_t* const d0 = d - sh;  // 16-byte aligned
+        const int end = sh + n;
+        const bool half = UNIT == 2 && (sh & 2) != 0;
+        for (int c = 16 * lane; c < end; c += 512) {
+            uint4 v = lds128(buf + c);
+            if (half) {
+                const uint32_t b = c ? lds32(buf + c - 4) : 0u;
+                v = make_uint4(__byte_perm(b, v.x, 0x5432), __byte_perm(v.x, v.y, 0x5432),
+                               __byte_perm(v.y, v.z, 0x5432), __byte_perm(v.z, v.w, 0x5432));
+            }
+            if (c >= sh && c + 16 <= end) {
+                __stcs((uint4*)(d0 + c), v);
+            } else {  // the first and the last chunk
+                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int i = b + k * 32 + lane;
-            if (i < cnt) v[k] = __ldcs((const T*)src + i);
+                for (int h = 0; h < 8; ++h) {
+                    const int q = c + 2 * h;
+                    if (q >= sh && q < end) *(uint16_t*)(d0 + q) = (uint16_t)(w[h >> 1] >> (16 * (h & 1)));
+                }
+            }
         }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int i = b + k * 32 + lane;
-            if (i < cnt) __stcs((T*)dst + i, v[k]);
-        }
+        __syncwarp();  // the buffer is free
     }
-    __syncwarp();
     for (int l = lane; l < (len + 127) >> 7; l += 32)
         asm volatile("discard.global.L2 [%0], 128;" ::"l"(__cvta_generic_to_global(src + 128 * l))
                      : "memory");
@@ -368,10 +371,9 @@ __device__ __forceinline__ int enc_tile(const Launch& P, const Item& it, unsigne
     const int un = ue0 < n ? (int)min(n - ue0, (unsigned long long)(U * 32)) : 0;  // unit elements
     const TX* const xp = (const TX*)it.x + ue0;
     const bool vec = ((uintptr_t)xp & 15u) == 0;
-    if (un > 0) {
-        if (lane == 0) prefetch_l2(xp, (unsigned)un * (unsigned)sizeof(TX));
-        stage_in<TX>(xp, min(un, GELEMS), vec, bufs);
-    }
+    // (requesting the whole unit into L2 here cost 5 of 152 us on the 512^3
+    // field: it displaces ring lines)
+    if (un > 0) stage_in<TX>(xp, min(un, GELEMS), vec, bufs);
     float two_eb_in = 0.0f;
     if (do_cin) {
         if (tid == 0) {
@@ -506,7 +508,7 @@ __device__ __forceinline__ int enc_tile(const Launch& P, const Item& it, unsigne
 template <int LOG2L, int U, bool HAS_CIN, bool HEADS = false>
 __device__ __forceinline__ void fin_tile(const Launch& P, const Item& it, unsigned item_idx,
                                          unsigned tile_in_item, unsigned g, const TileSlot& S,
-                                         const uint8_t* seg, const uint8_t* wb)
+                                         const uint8_t* seg, const uint8_t* wb, unsigned buf)
 {
     constexpr int L = 1 << LOG2L;
     constexpr int PB = L / 8;
@@ -532,7 +534,7 @@ __device__ __forceinline__ void fin_tile(const Launch& P, const Item& it, unsign
     const unsigned long long end = base + payload;  // unpadded end of this tile's payload
     if (base + payload <= cap) {
         if (dcheck(P.ctl, S.segsz[warp] <= seg_bytes(U), g))
-            ring_copy<PB>(out + base + segoff, seg, S.segsz[warp]);
+            ring_copy<PB>(out + base + segoff, seg, S.segsz[warp], buf);
     } else if (tid == 0) {
         fail(P.ctl, ZC_ERR_CAPACITY, g);
     }
@@ -762,7 +764,7 @@ __device__ __forceinline__ void resolve_slot(const Launch& P, TileSlot& S, unsig
 // publishes its tiles in ticket order, so the chain always advances.  The
 // last CTA to finish advances the launch generation.
 //   enc(item, index, tile in item, segment, width bytes, stage, slot, shared) -> unit size
-//   fin(item, index, tile in item, ticket, slot, segment, width bytes)
+//   fin(item, index, tile in item, ticket, slot, segment, width bytes, free group buffer)
 // Barrier protocol per tile in slot s: the encoder warps arrive on BAR_ENC + s
 // after encoding it, the resolver waits there, resolves it and arrives on
 // BAR_RES + s, where the encoder warps wait NS - 1 tiles later before
@@ -810,7 +812,7 @@ __device__ __forceinline__ void enc_pipeline(const Launch& P, const Src& src, En
             const TileSlot& Q = slots[q];
             if (Q.ok) {
                 const Item it = src.get(Q.item);
-                fin(it, Q.item, Q.tile, Q.g, Q, seg_of(q), wb_of(q));
+                fin(it, Q.item, Q.tile, Q.g, Q, seg_of(q), wb_of(q), bufs);
             }
         };
         int s = 0;
@@ -884,7 +886,7 @@ __global__ void __launch_bounds__(ENC_THREADS, ENC_CTAS_PER_SM) k_compress(const
             return enc_tile<LOG2L, U, false, TX, HEADS>(P, it, idx, t, seg, wb, bufs, S, es);
         },
         [&](const Item& it, unsigned idx, unsigned t, unsigned g, const TileSlot& S,
-            const uint8_t* seg, const uint8_t* wb) { fin_tile<LOG2L, U, false, HEADS>(P, it, idx, t, g, S, seg, wb); });
+            const uint8_t* seg, const uint8_t* wb, unsigned buf) { fin_tile<LOG2L, U, false, HEADS>(P, it, idx, t, g, S, seg, wb, buf); });
 }
 
 template <int LOG2L, int U, typename TX>
@@ -898,7 +900,7 @@ __global__ void __launch_bounds__(ENC_THREADS, ENC_CTAS_PER_SM) k_scatter(const 
             return enc_tile<LOG2L, U, false, TX>(P, it, idx, t, seg, wb, bufs, S, es);
         },
         [&](const Item& it, unsigned idx, unsigned t, unsigned g, const TileSlot& S,
-            const uint8_t* seg, const uint8_t* wb) { fin_tile<LOG2L, U, false>(P, it, idx, t, g, S, seg, wb); });
+            const uint8_t* seg, const uint8_t* wb, unsigned buf) { fin_tile<LOG2L, U, false>(P, it, idx, t, g, S, seg, wb, buf); });
 }
 
 template <int LOG2L, int U>
@@ -911,7 +913,7 @@ __global__ void __launch_bounds__(ENC_THREADS, ENC_CTAS_PER_SM) k_reduce(const L
             return enc_tile<LOG2L, U, true, float>(P, it, idx, t, seg, wb, bufs, S, es);
         },
         [&](const Item& it, unsigned idx, unsigned t, unsigned g, const TileSlot& S,
-            const uint8_t* seg, const uint8_t* wb) { fin_tile<LOG2L, U, true>(P, it, idx, t, g, S, seg, wb); });
+            const uint8_t* seg, const uint8_t* wb, unsigned buf) { fin_tile<LOG2L, U, true>(P, it, idx, t, g, S, seg, wb, buf); });
 }
 
 // ---- batched compression -----------------------------------------------------
@@ -944,12 +946,12 @@ __global__ void __launch_bounds__(ENC_THREADS, ENC_CTAS_PER_SM) k_batch(const La
             }
         },
         [&](const Item& it, unsigned idx, unsigned t, unsigned g, const TileSlot& S,
-            const uint8_t* seg, const uint8_t* wb) {
+            const uint8_t* seg, const uint8_t* wb, unsigned buf) {
             switch (it.log2L) {
-            case 4: fin_tile<4, U, false>(P, it, idx, t, g, S, seg, wb); break;
-            case 5: fin_tile<5, U, false>(P, it, idx, t, g, S, seg, wb); break;
-            case 6: fin_tile<6, U, false>(P, it, idx, t, g, S, seg, wb); break;
-            case 7: fin_tile<7, U, false>(P, it, idx, t, g, S, seg, wb); break;
+            case 4: fin_tile<4, U, false>(P, it, idx, t, g, S, seg, wb, buf); break;
+            case 5: fin_tile<5, U, false>(P, it, idx, t, g, S, seg, wb, buf); break;
+            case 6: fin_tile<6, U, false>(P, it, idx, t, g, S, seg, wb, buf); break;
+            case 7: fin_tile<7, U, false>(P, it, idx, t, g, S, seg, wb, buf); break;
             default: fin_raw<U>(P, it, idx, t, g, S); break;
             }
         });
