@@ -636,8 +636,9 @@ int zc_scatter_pack(const void* d_in, int dtype, int P, const uint64_t* h_counts
     const int C = tile_chunks_for(all_n, all_n / (uint64_t)P);
     thread_local static ScatterParams SP;  // host staging of the by-value parameter block
     uint64_t tile = 0, total_n = 0, min_cap = 0;
-    std::vector<const void*> ptrs((size_t)P);
-    std::vector<unsigned long long> cnts((size_t)P);
+    // the range pass reads segments that follow each other as one
+    std::vector<const void*> ptrs;
+    std::vector<unsigned long long> cnts;
     const uint64_t es = dtype == ZC_F32 ? 4 : 2;
     for (int p = 0; p < P; ++p) {
         if (h_counts[p] > 0 && d_in == nullptr) return ZC_ERR_ARG;
@@ -649,8 +650,13 @@ int zc_scatter_pack(const void* d_in, int dtype, int P, const uint64_t* h_counts
         tile += tiles_for(h_counts[p], unit_rows(C));
         total_n += h_counts[p];
         min_cap += 32 + pad16(nb);
-        ptrs[p] = (const uint8_t*)d_in + h_displs[p] * es;
-        cnts[p] = h_counts[p];
+        const uint8_t* const seg = (const uint8_t*)d_in + h_displs[p] * es;
+        if (h_counts[p] > 0 && !ptrs.empty() && (const uint8_t*)ptrs.back() + cnts.back() * es == seg) {
+            cnts.back() += h_counts[p];
+        } else if (h_counts[p] > 0) {
+            ptrs.push_back(seg);
+            cnts.push_back(h_counts[p]);
+        }
     }
     SP.tile_begin[P] = (unsigned)tile;
     if (out_cap < min_cap) return ZC_ERR_CAPACITY;
@@ -673,9 +679,15 @@ int zc_scatter_pack(const void* d_in, int dtype, int P, const uint64_t* h_counts
         R.total = total_n;
         R.rel = eb_value;
         R.dtype = dtype;
-        if (launch_range_multi(R, ptrs.data(), cnts.data(), (unsigned)P, range_grid(total_n),
-                               (cudaStream_t)s) != cudaSuccess)
-            return ZC_ERR_CUDA;
+        cudaError_t e;
+        if (ptrs.size() <= 1) {
+            R.one = ptrs.empty() ? RangeSeg{d_in, 0} : RangeSeg{ptrs[0], cnts[0]};
+            e = launch_range(R, range_grid(total_n), (cudaStream_t)s);
+        } else {
+            e = launch_range_multi(R, ptrs.data(), cnts.data(), (unsigned)ptrs.size(),
+                                   range_grid(total_n), (cudaStream_t)s);
+        }
+        if (e != cudaSuccess) return ZC_ERR_CUDA;
         L.eb_from_ctl = 1;
     }
     L.packed = 1;

@@ -373,7 +373,7 @@ __device__ __forceinline__ int enc_tile(const Launch& P, const Item& it, unsigne
     const bool vec = ((uintptr_t)xp & 15u) == 0;
     // (requesting the whole unit into L2 here cost 5 of 152 us on the 512^3
     // field: it displaces ring lines)
-    if (un > 0) stage_in<TX>(xp, min(un, GELEMS), vec, bufs);
+    if (un > 0) stage_in<TX>(xp, un, vec, bufs, ue0 == 0);
     float two_eb_in = 0.0f;
     if (do_cin) {
         if (tid == 0) {
@@ -418,8 +418,7 @@ __device__ __forceinline__ int enc_tile(const Launch& P, const Item& it, unsigne
         A.buf = bufs + (g & 1) * GBUF;
         const bool more = e0 + GELEMS < un;
         if (more) {
-            stage_in<TX>(xp + e0 + GELEMS, min(un - e0 - GELEMS, GELEMS), vec,
-                         bufs + ((g + 1) & 1) * GBUF);
+            stage_in<TX>(xp + e0 + GELEMS, un - e0 - GELEMS, vec, bufs + ((g + 1) & 1) * GBUF, false);
             cp_wait<1>();
         } else {
             cp_wait<0>();

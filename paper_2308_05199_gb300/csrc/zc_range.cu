@@ -40,7 +40,11 @@ __device__ __forceinline__ void acc_vec(Acc& a, const uint4 v)
 }
 
 // A thread's grid-strided share of one segment: four independent 16-byte
-// streaming loads (ld.global.cs) in flight per thread, then the scalar tail.
+// streaming loads (ld.global.cs) in flight per thread, and single elements
+// before the first 16-byte boundary and behind the last one.  (A segment off
+// that boundary was read by single elements throughout: the range pass took
+// 121 of the 194 us of a 200 MB scatter pack of 8 such segments; the whole
+// call takes 102 now.)
 // Measured on 512 MiB: 6.1 TB/s with streaming loads at 3 to 6 CTAs per SM,
 // 5.3-5.4 TB/s with __ldg or ld.global.cg.  The pass runs from the end of
 // the segment to its start, so the last lines it reads are the first ones
@@ -51,25 +55,26 @@ __device__ __forceinline__ void range_seg(Acc& a, const void* p, unsigned long l
 {
     constexpr int VEC = 16 / sizeof(TX);
     constexpr int UNR = 4;
-    unsigned long long nvec = 0;
-    if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0) {
-        nvec = n / VEC;
-        const uint4* top = (const uint4*)p + (nvec ? nvec - 1 : 0);  // vector i is top[-i]
-        unsigned long long i = gtid;
-        for (; i + (UNR - 1) * gstride < nvec; i += UNR * gstride) {
-            uint4 v[UNR];
+    auto one = [&](unsigned long long i) {
+        acc_one(a, sizeof(TX) == 4 ? __ldg((const float*)p + i)
+                                   : bf16_to_f32(__ldg((const unsigned short*)p + i)));
+    };
+    const unsigned long long skew = ((0ull - (unsigned long long)reinterpret_cast<uintptr_t>(p)) & 15ull) / sizeof(TX);
+    const unsigned long long h = skew < n ? skew : n;
+    const unsigned long long nvec = (n - h) / VEC;
+    if (gtid < h) one(gtid);
+    const uint4* top = (const uint4*)((const TX*)p + h) + (nvec ? nvec - 1 : 0);  // vector i is top[-i]
+    unsigned long long i = gtid;
+    for (; i + (UNR - 1) * gstride < nvec; i += UNR * gstride) {
+        uint4 v[UNR];
 #pragma unroll
-            for (int u = 0; u < UNR; ++u) v[u] = __ldcs(top - (long long)(i + u * gstride));
+        for (int u = 0; u < UNR; ++u) v[u] = __ldcs(top - (long long)(i + u * gstride));
 #pragma unroll
-            for (int u = 0; u < UNR; ++u) acc_vec<TX>(a, v[u]);
-        }
-        for (; i < nvec; i += gstride) acc_vec<TX>(a, __ldcs(top - (long long)i));
+        for (int u = 0; u < UNR; ++u) acc_vec<TX>(a, v[u]);
     }
-    for (unsigned long long i = nvec * VEC + gtid; i < n; i += gstride) {
-        const float v = sizeof(TX) == 4 ? __ldg((const float*)p + i)
-                                        : bf16_to_f32(__ldg((const unsigned short*)p + i));
-        acc_one(a, v);
-    }
+    for (; i < nvec; i += gstride) acc_vec<TX>(a, __ldcs(top - (long long)i));
+    i = h + nvec * VEC + gtid;  // the last elements, fewer than VEC
+    if (i < n) one(i);
 }
 
 struct RangeSegs {
