@@ -140,6 +140,8 @@ int ws_view(void* ws, size_t bytes, WsView& v)
 // Width scans over at least this many items find a chunk's item in a map
 // (one extra launch); fewer items are searched (at most 8 dependent loads).
 constexpr int CHUNK_MAP_ITEMS = 256;
+// The fused step finds a tile's item by search up to this many items.
+constexpr int SEARCH_ITEMS = 16;
 
 // SM count of the current device (queried once per device).
 int sm_count()
@@ -259,6 +261,15 @@ cudaError_t launch_batch(int C, const Launch& P, unsigned grid, cudaStream_t s)
 }
 
 inline uint64_t elem_bytes(int dtype) { return dtype == ZC_F32 ? 4 : 2; }
+
+// Largest item (in decode tiles) of a batched decompression that goes without
+// width-scan chunks.
+unsigned dec_local_tiles(int n_msgs, const zc_message* msgs)
+{
+    uint64_t tiles = 0;
+    for (int i = 0; i < n_msgs; ++i) tiles += tiles_for(msgs[i].n, DEC_U);
+    return tiles <= LOCAL_LAUNCH_TILES ? DEC_LOCAL_FEW_TILES : DEC_LOCAL_TILES;
+}
 
 }  // namespace
 
@@ -435,7 +446,7 @@ int zc_decompress(const void* d_cmp, size_t cmp_cap, void* d_out, uint64_t n, in
     int st = ws_view(d_ws, ws_bytes, w);
     if (st) return st;
     const uint64_t tiles = tiles_for(n, DEC_U);
-    const uint64_t chunks = chunks_for(tiles);
+    const uint64_t chunks = tiles <= DEC_LOCAL_SINGLE_TILES ? 0 : chunks_for(tiles);
     if (tiles * NWARPS > w.cap || tiles > 0x7fffffffull) return ZC_ERR_WORKSPACE;
     Launch P = base_launch(w);
     Item& it = P.one;
@@ -449,9 +460,9 @@ int zc_decompress(const void* d_cmp, size_t cmp_cap, void* d_out, uint64_t n, in
     P.n_items = 1;
     P.urows = DEC_U;
     P.total_tiles = (unsigned)chunks;
-    if (launch_wscan(P, (unsigned)chunks, (cudaStream_t)s) != cudaSuccess) return ZC_ERR_CUDA;
+    if (chunks > 0 && launch_wscan(P, (unsigned)chunks, (cudaStream_t)s) != cudaSuccess) return ZC_ERR_CUDA;
     P.total_tiles = (unsigned)tiles;
-    return cuda_status(launch_decompress(P, (unsigned)tiles, (cudaStream_t)s, true));
+    return cuda_status(launch_decompress(P, (unsigned)tiles, (cudaStream_t)s, chunks > 0));
 }
 
 int zc_reduce_step(const void* d_cmp_in, size_t cmp_in_cap, const float* d_local, uint64_t n,
@@ -473,7 +484,7 @@ int zc_reduce_step(const void* d_cmp_in, size_t cmp_in_cap, const float* d_local
     if (st) return st;
     const int C = tile_chunks_for(n, n);
     const uint64_t tiles = tiles_for(n, unit_rows(C));
-    const uint64_t chunks = chunks_for(tiles);
+    const uint64_t chunks = tiles <= LOCAL_LAUNCH_TILES && nb <= RED_LOCAL_BLOCKS ? 0 : chunks_for(tiles);
     if (tiles * NWARPS > w.cap || tiles > 0x7fffffffull) return ZC_ERR_WORKSPACE;
     Launch P = base_launch(w);
     Item& it = P.one;
@@ -493,7 +504,7 @@ int zc_reduce_step(const void* d_cmp_in, size_t cmp_in_cap, const float* d_local
     it.out_dtype = ZC_F32;
     P.n_items = 1;
     P.urows = unit_rows(C);
-    if (d_cmp_in != nullptr) {
+    if (d_cmp_in != nullptr && chunks > 0) {
         P.total_tiles = (unsigned)chunks;
         if (launch_wscan(P, (unsigned)chunks, (cudaStream_t)s) != cudaSuccess) return ZC_ERR_CUDA;
     }
@@ -522,7 +533,8 @@ int zc_plan_reduce(zc_plan* plan, int P, const zc_reduce_item* h_items, double e
     for (int r = 0; r < P; ++r) total_n += h_items[r].n;
     const int C = tile_chunks_for(total_n, total_n / (uint64_t)P);
     std::vector<Item> items((size_t)P);
-    uint64_t tile = 0, chunk = 0;
+    uint64_t tile = 0, chunk = 0, all_tiles = 0;
+    for (int r = 0; r < P; ++r) all_tiles += tiles_for(h_items[r].n, unit_rows(C));
     int has_cin = 0;
     for (int r = 0; r < P; ++r) {
         const zc_reduce_item& h = h_items[r];
@@ -550,7 +562,9 @@ int zc_plan_reduce(zc_plan* plan, int P, const zc_reduce_item* h_items, double e
         it.tile_begin = (unsigned)tile;
         it.ntiles = (unsigned)tiles_for(h.n, unit_rows(C));
         it.chunk_begin = (unsigned)chunk;
-        it.nchunks = (unsigned)chunks_for(it.ntiles);
+        it.nchunks = all_tiles <= LOCAL_LAUNCH_TILES && nb <= RED_LOCAL_BLOCKS
+                         ? 0u
+                         : (unsigned)chunks_for(it.ntiles);
         it.x_dtype = ZC_F32;
         it.out_dtype = ZC_F32;
         tile += it.ntiles;
@@ -585,7 +599,8 @@ int zc_reduce_step_batch(const zc_plan* plan, void* d_ws, size_t ws_bytes, zc_st
     P.items = (const Item*)plan->d_table;
     P.n_items = (unsigned)plan->n_items;
     P.urows = unit_rows(C);
-    if (plan->has_input) {
+    const bool scan = plan->has_input != 0 && plan->total_chunks > 0;
+    if (scan) {
         P.total_tiles = (unsigned)plan->total_chunks;
         if (plan->n_items >= CHUNK_MAP_ITEMS) {
             // chunk -> item map for the width scan (the tile map below reuses its space)
@@ -603,15 +618,19 @@ int zc_reduce_step_batch(const zc_plan* plan, void* d_ws, size_t ws_bytes, zc_st
     if (grid == 0) return ZC_ERR_WORKSPACE;
     // each launch of the step is dependent on the one before it: the tile
     // map is built while the width scan runs, the fused kernel's CTAs become
-    // resident while the map finishes (both wait for their inputs)
-    if (plan->n_items > 1) {
+    // resident while the map finishes (both wait for their inputs).  Few
+    // items are searched instead: one thread's few loads per tile, from L1
+    // after its CTA's first tile, against a launch of about 4 us
+    // (the five-rank recursive
+    // doubling of 1M elements: 142 us with maps, 139 us without).
+    if (plan->n_items > SEARCH_ITEMS) {
         if (launch_tile_map(P.items, P.n_items, P.total_tiles, w.tile_map, (cudaStream_t)s,
-                            false, plan->has_input != 0) != cudaSuccess)
+                            false, scan) != cudaSuccess)
             return ZC_ERR_CUDA;
         P.tile_map = w.tile_map;
         P.dep = 1;
     } else {
-        P.dep = plan->has_input != 0;
+        P.dep = scan;
     }
     return cuda_status(launch_reduce_any(lg, C, P, (unsigned)grid, (cudaStream_t)s));
 }
@@ -829,6 +848,7 @@ int zc_plan_decompress_batch(zc_batch* plan, int n_msgs, const zc_message* h_msg
         return ZC_ERR_ARG;
     std::vector<Item> items((size_t)n_msgs);
     uint64_t tile = 0, chunk = 0;
+    const unsigned local = dec_local_tiles(n_msgs, h_msgs);
     for (int i = 0; i < n_msgs; ++i) {
         const zc_message& m = h_msgs[i];
         if (!dtype_ok(m.dtype) || (m.n > 0 && m.out == nullptr) ||
@@ -842,7 +862,7 @@ int zc_plan_decompress_batch(zc_batch* plan, int n_msgs, const zc_message* h_msg
         it.tile_begin = (unsigned)tile;
         it.ntiles = (unsigned)tiles_for(m.n, DEC_U);
         it.chunk_begin = (unsigned)chunk;
-        it.nchunks = it.ntiles <= DEC_LOCAL_TILES ? 0u : (unsigned)chunks_for(it.ntiles);
+        it.nchunks = it.ntiles <= local ? 0u : (unsigned)chunks_for(it.ntiles);
         it.x_dtype = m.dtype;
         it.out_dtype = m.dtype;
         tile += it.ntiles;
@@ -876,6 +896,7 @@ int zc_plan_decompress_streams(zc_batch* plan, int n_msgs, const void* const* h_
         return ZC_ERR_ARG;
     std::vector<Item> items((size_t)n_msgs);
     uint64_t tile = 0, chunk = 0;
+    const unsigned local = dec_local_tiles(n_msgs, h_msgs);
     for (int i = 0; i < n_msgs; ++i) {
         const zc_message& m = h_msgs[i];
         if (!dtype_ok(m.dtype) || (m.n > 0 && m.out == nullptr) ||
@@ -891,7 +912,7 @@ int zc_plan_decompress_streams(zc_batch* plan, int n_msgs, const void* const* h_
         it.tile_begin = (unsigned)tile;
         it.ntiles = (unsigned)tiles_for(m.n, DEC_U);
         it.chunk_begin = (unsigned)chunk;
-        it.nchunks = it.ntiles <= DEC_LOCAL_TILES ? 0u : (unsigned)chunks_for(it.ntiles);
+        it.nchunks = it.ntiles <= local ? 0u : (unsigned)chunks_for(it.ntiles);
         it.x_dtype = m.dtype;
         it.out_dtype = m.dtype;
         tile += it.ntiles;

@@ -31,6 +31,23 @@ constexpr int DEC_U = 64;              // rows per warp unit of the decompressor
 // Batched decompression: items of at most this many decode tiles get no
 // width-scan chunks; their decoder CTAs find the unit offsets themselves.
 constexpr unsigned DEC_LOCAL_TILES = 4;
+// In launches of at most this many tiles (about two per resident CTA) that
+// holds for larger items too: up to DEC_LOCAL_FEW_TILES decode tiles, and in
+// the fused step up to RED_LOCAL_BLOCKS blocks (width bytes).  Few CTAs then
+// each read at most 128 KiB of width bytes, from L2, where the scan would be a
+// launch in front of a short one (the five-rank recursive doubling of 1M
+// elements: 139 us with four scans, 118 us without).
+constexpr unsigned LOCAL_LAUNCH_TILES = 1024;
+constexpr unsigned DEC_LOCAL_FEW_TILES = 128;
+constexpr unsigned RED_LOCAL_BLOCKS = 1u << 16;
+// Decompression of one stream: up to this many decode tiles (16384 elements
+// each) every CTA sums the width bytes before its tile itself, 16 bytes per
+// thread and load, and there is no width scan: the scan costs a launch and
+// some seven dependent round trips, the sums of a last tile here at most
+// 256 KiB / 4 KiB = 64 loads per thread, four in flight.  Measured with / without
+// the scan: 2^21 elements 10.8 / 7.5 us at L = 32, 12.6 / 9.2 at L = 16; 2^22 elements
+// 13.7 / 10.5 and 15.8 / 13.5; 2^23 elements 17.4 / 20.5 and 20.3 / 29.0.
+constexpr unsigned DEC_LOCAL_SINGLE_TILES = 256;
 
 // Rows per warp unit of an encoder tile of `chunks` 2048-element chunks.
 __host__ __device__ constexpr int unit_rows(int chunks) { return chunks * 8; }
@@ -215,6 +232,31 @@ __device__ __forceinline__ uint32_t load_widths(const uint8_t* cin, unsigned lon
                       : (uint32_t)__ldg(cin + 32 + b);
 }
 
+// Planes of 16 width bytes at byte b of a stream's width array: the sum of
+// w + 1 over the nonzero widths, four bytes at a time (a width above the
+// format's counts as none and is reported when `ctl` is set).
+__device__ __forceinline__ int planes16(const uint4& v, Ctl* ctl, unsigned long long b)
+{
+    const unsigned w[4] = {v.x, v.y, v.z, v.w};
+    unsigned sum = 0u, bad = 0u;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        sum = __dp4a(w[q], 0x01010101u, sum);
+        sum += __popc((w[q] + 0x7f7f7f7fu) & 0x80808080u);          // bytes that are not 0
+        bad |= w[q] | (w[q] + 0x01010101u * (127 - ZC_MAX_WIDTH));  // bit 7: above the largest
+    }
+    if ((bad & 0x80808080u) == 0u) return (int)sum;
+    sum = 0u;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        for (int k = 0; k < 4; ++k) {
+            const int x = (w[q] >> (8 * k)) & 0xff;
+            if (x <= ZC_MAX_WIDTH) sum += planes_of(x);
+            else if (ctl != nullptr) fail(ctl, ZC_ERR_FORMAT, b + 4 * q + k);
+        }
+    return (int)sum;
+}
+
 // ---- encoder tiles -------------------------------------------------------------
 // An encoder CTA runs two kinds of warps.  Its NWARPS encoder warps take tiles
 // in ticket order and encode each of the tile's warp units into the CTA's ring
@@ -330,7 +372,53 @@ struct EncShared {
     int abort;     // 1: unusable workspace (the CTA does nothing), 2: no usable bound
     int hdr_bad;   // fused ring step: the tile's input stream failed its check
     float eb_in;   // its bound
+    unsigned pre[NWARPS], own[NWARPS];  // planes before the tile and of its units (items without a width scan)
 };
+
+// Payload offset of this warp's unit of a received stream without a width
+// scan: the encoder warps of the CTA sum the width bytes before the tile and
+// of its units (16 bytes per thread and load).  The item's last tile checks
+// the total against the header's payload size, as the scan does.
+template <int LOG2L, int U>
+__device__ __forceinline__ unsigned long long tile_unit_offset(const Item& it, unsigned t, Ctl* ctl,
+                                                               unsigned item_idx, EncShared& es)
+{
+    constexpr unsigned BPU = U * 32 >> LOG2L;  // blocks per unit: 8, or a multiple of 16
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const unsigned wbytes = (unsigned)ceil16((it.n + (1ull << LOG2L) - 1) >> LOG2L);
+    const uint8_t* const w = it.cin + 32;
+    const unsigned t0 = min(t * NWARPS * BPU, wbytes);  // a multiple of 16
+    unsigned pre = 0u, own = 0u;
+#pragma unroll 4
+    for (unsigned o = 16 * tid; o < t0; o += 16 * NTHREADS) pre += planes16(__ldg((const uint4*)(w + o)), nullptr, 0ull);
+    const unsigned u0 = (t * NWARPS + warp) * BPU;
+    if (BPU == 8) {
+        if (lane == 0 && u0 < wbytes) {
+            const uint2 v = __ldg((const uint2*)(w + u0));
+            own = planes16(make_uint4(v.x, v.y, 0u, 0u), nullptr, 0ull);
+        }
+    } else {
+        const unsigned o = u0 + 16 * lane;
+        if (lane < (int)(BPU / 16) && o < wbytes) own = planes16(__ldg((const uint4*)(w + o)), nullptr, 0ull);
+    }
+    pre = __reduce_add_sync(FULL, pre);
+    own = __reduce_add_sync(FULL, own);
+    if (lane == 0) {
+        es.pre[warp] = pre;
+        es.own[warp] = own;
+    }
+    bar_sync_n(BAR_ENCW, NTHREADS);
+    unsigned off = 0u, total = 0u;
+#pragma unroll
+    for (int v = 0; v < NWARPS; ++v) {
+        off += es.pre[v] + (v < warp ? es.own[v] : 0u);
+        total += es.pre[v] + es.own[v];
+    }
+    constexpr unsigned long long PB = (1ull << LOG2L) / 8;
+    if (t + 1 == it.ntiles && tid == 0 && total * PB != __ldg((const unsigned long long*)it.cin + 3))
+        fail(ctl, ZC_ERR_FORMAT, item_idx);
+    return off * PB;
+}
 
 // Encoder warp `warp`'s unit of one tile: quantize, delta-code and bit-plane
 // pack its U rows, 32 rows at a time (zc_rows.cuh), into its ring segment
@@ -390,7 +478,7 @@ __device__ __forceinline__ int enc_tile(const Launch& P, const Item& it, unsigne
         }
         two_eb_in = __fadd_rn(es.eb_in, es.eb_in);
     }
-    if (un == 0) return 0;
+    if (un == 0 && !(do_cin && it.nchunks == 0)) return 0;
     EncArgs A;
     A.eb = it.eb;
     A.two_eb = it.two_eb;
@@ -405,8 +493,13 @@ __device__ __forceinline__ int enc_tile(const Launch& P, const Item& it, unsigne
     unsigned long long pos = 0ull;  // received stream: payload position of the group
     uint32_t wv = 0u;               // and its width byte(s) of this lane's row
     if (do_cin) {
-        const unsigned slot = S.g * NWARPS + warp;
-        pos = 32ull + wbytes + (dcheck(ctl, slot < P.ws_cap, slot) ? P.offs[slot] : 0ull);
+        if (it.nchunks == 0) {
+            pos = 32ull + wbytes + tile_unit_offset<LOG2L, U>(it, tile_in_item, ctl, item_idx, es);
+        } else {
+            const unsigned slot = S.g * NWARPS + warp;
+            pos = 32ull + wbytes + (dcheck(ctl, slot < P.ws_cap, slot) ? P.offs[slot] : 0ull);
+        }
+        if (un == 0) return 0;  // (its warp took part in the tile's sums)
         wv = load_widths<LOG2L>(it.cin, nb, ue0 >> LOG2L);
     }
     int err = 0;
@@ -1117,7 +1210,8 @@ __global__ void __launch_bounds__(GROUP_T) k_group_place(Item* items, unsigned n
 
 // ---- width scan: payload offset of every decode tile --------------------------
 // One CTA per chunk of WSCAN warp units of one item; thread i sums the plane
-// bytes of unit i from its width bytes; a CTA scan and a look-back over the
+// bytes of unit i from its width bytes, four 16-byte loads in flight (the first
+// one of a line brings the others' bytes to L1); a CTA scan and a look-back over the
 // item's chunks give every unit's payload offset (global decode slot = item
 // tile slot * NWARPS + unit in tile).  A multi-item launch finds a chunk's
 // item in P.tile_map, here the chunk -> item map (k_tile_map by chunk).
@@ -1126,36 +1220,40 @@ __global__ void __launch_bounds__(NTHREADS) k_wscan(const Launch P)
     __shared__ Smem sm;
     __shared__ int wsum[NWARPS];
     grid_dep_launch();  // the decoder after it may be launched now (it waits for the offsets)
-    if (threadIdx.x == 0) {
+    const unsigned modulus = P.total_tiles + gridDim.x - 1u;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // the first ticket is taken with the control block's words: one round trip
+    unsigned first = 0u;
+    if (tid == 0) {
+        first = atomicInc(&P.ctl->ticket, modulus);
         sm.E = ld_volatile_u32(&P.ctl->epoch) + 1u;
         sm.abort = ld_volatile_u32(&P.ctl->magic) != WS_MAGIC;
         if (sm.abort) fail(P.ctl, ZC_ERR_WORKSPACE, 0);
     }
-    __syncthreads();
-    if (sm.abort) return;
-    const unsigned modulus = P.total_tiles + gridDim.x - 1u;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    while (true) {
+    for (bool again = false;; again = true) {
         __syncthreads();
-        if (tid == 0) {
-            sm.ticket = atomicInc(&P.ctl->ticket, modulus);
+        if (warp == 0) {
+            const unsigned g = __shfl_sync(FULL, again && lane == 0 ? atomicInc(&P.ctl->ticket, modulus) : first, 0);
             unsigned it = 0;
-            if (P.items != nullptr && sm.ticket < P.total_tiles) {
+            if (P.items != nullptr && g < P.total_tiles) {
                 if (P.tile_map != nullptr) {
-                    it = P.tile_map[sm.ticket];  // the chunk map of this launch
-                } else {
-                    unsigned lo = 0, hi = P.n_items;
-                    while (hi - lo > 1) {
-                        const unsigned mid = (lo + hi) >> 1;
-                        if (P.items[mid].chunk_begin <= sm.ticket) lo = mid;
-                        else hi = mid;
+                    it = P.tile_map[g];  // the chunk map of this launch
+                } else {  // the last item that begins at or before g, 32 candidates per round trip
+                    for (unsigned i0 = 0; i0 < P.n_items; i0 += 32) {
+                        const bool le = i0 + lane < P.n_items && P.items[i0 + lane].chunk_begin <= g;
+                        const unsigned m = __ballot_sync(FULL, le);
+                        if (m) it = i0 + 31 - __clz(m);
+                        if (m != FULL) break;
                     }
-                    it = lo;
                 }
             }
-            sm.item = it;
+            if (lane == 0) {
+                sm.ticket = g;
+                sm.item = it;
+            }
         }
         __syncthreads();
+        if (sm.abort) return;
         const unsigned c = sm.ticket;
         if (c >= P.total_tiles) break;
         Item it = P.items != nullptr ? P.items[sm.item] : P.one;
@@ -1172,35 +1270,26 @@ __global__ void __launch_bounds__(NTHREADS) k_wscan(const Launch P)
         const unsigned long long ntile = (unsigned long long)it.ntiles * NWARPS;  // units
         const unsigned long long k = (unsigned long long)chunk * WSCAN + tid;    // unit in item
         const int bpt = (P.urows * 32) >> lgb;                                   // blocks per unit
+        // bpt is 8 (32-row units at L = 128) or a power of two from 16 on
+        const unsigned long long b0 = k * bpt, wend = ceil16(nb);
         int sum = 0;
-        if (k < ntile) {
-            const unsigned long long b0 = k * bpt;
-            const uint8_t* w = it.cin + 32;
-            // bpt is 8 (32-row units at L = 128) or a multiple of 16
-            const int step = bpt < 16 ? 8 : 16;
-            for (int i = 0; i < bpt; i += step) {
-                if (b0 + i >= ceil16(nb)) break;
-                unsigned ws[4] = {0u, 0u, 0u, 0u};
-                if (step == 16) {
-                    const uint4 v = __ldg((const uint4*)(w + b0 + i));
-                    ws[0] = v.x;
-                    ws[1] = v.y;
-                    ws[2] = v.z;
-                    ws[3] = v.w;
-                } else {
-                    const uint2 v = __ldg((const uint2*)(w + b0 + i));
-                    ws[0] = v.x;
-                    ws[1] = v.y;
+        if (k < ntile && b0 < wend) {
+            const uint8_t* const w = it.cin + 32 + b0;
+            if (bpt == 8) {
+                const uint2 v = __ldg((const uint2*)w);
+                sum = planes16(make_uint4(v.x, v.y, 0u, 0u), P.ctl, b0);
+            } else {
+                const int nv = (int)min((unsigned long long)bpt, wend - b0) / 16;
+                for (int i = 0; i < nv; i += 4) {
+                    uint4 v[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        v[q] = i + q < nv ? __ldg((const uint4*)w + i + q) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) sum += planes16(v[q], P.ctl, b0 + 16 * (i + q));
                 }
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        const int wv = (ws[q] >> (8 * b)) & 0xff;
-                        if (wv > ZC_MAX_WIDTH) fail(P.ctl, ZC_ERR_FORMAT, b0 + i + 4 * q + b);
-                        else sum += planes_of(wv) * PB;
-                    }
             }
+            sum *= PB;
         }
         int tot;
         const int ex = warp_excl_scan(sum, lane, tot);
@@ -1337,65 +1426,56 @@ __device__ __forceinline__ void unit_decode(const Launch& P, const Item& it, uns
     cp_wait<0>();
 }
 
-// Items of at most DEC_LOCAL_TILES decode tiles (planned with no width-scan
-// chunks) need no width scan: the decoder CTA of tile t sums the plane bytes
-// of the item's blocks before its tile itself (at most DEC_LOCAL_TILES - 1
-// tiles' width bytes) and its warps' units (one value per warp), which gives
-// every warp its unit's payload offset; the item's last tile checks the total
-// against the header's payload size, as the width scan does.  Called by every
-// thread of the CTA (coded streams only: lg >= 4).
+// Items planned with no width-scan chunks (small ones): the decoder CTA of tile
+// t sums the plane bytes of the item's blocks before its tile itself and its
+// warps' units (one value per warp), which gives every warp its unit's payload
+// offset; the item's last tile checks the total against the header's payload
+// size, as the width scan does.  Called by every thread of the CTA (coded
+// streams only: lg >= 4).
 __device__ __forceinline__ unsigned long long local_unit_offset(const Item& it, int lg, unsigned t,
                                                                 Ctl* ctl, unsigned item_idx)
 {
-    __shared__ unsigned long long s_pre[NWARPS], s_own[NWARPS];
+    __shared__ unsigned s_pre[NWARPS], s_own[NWARPS];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int lgb = lg & 7;
     const unsigned long long PB = (1ull << lgb) / 8;
     const unsigned long long nb = (it.n + (1ull << lgb) - 1) >> lgb;
-    const unsigned long long bpu = (unsigned long long)(DEC_U * 32) >> lgb;  // blocks per unit
-    const uint8_t* w = it.cin + 32;
-    auto bytes_of = [&](unsigned long long b) -> unsigned long long {
-        const int wv = __ldg(w + b);
-        return wv > ZC_MAX_WIDTH ? 0ull : (unsigned long long)planes_of(wv) * PB;
-    };
-    const unsigned long long pre_end = min((unsigned long long)t * NWARPS * bpu, nb);
-    unsigned long long pre = 0ull;
-    for (unsigned long long b = tid; b < pre_end; b += NTHREADS) pre += bytes_of(b);
-    const unsigned long long u_lo = ((unsigned long long)t * NWARPS + warp) * bpu;
-    const unsigned long long u_hi = min(u_lo + bpu, nb);
-    unsigned long long own = 0ull;
-    for (unsigned long long b = u_lo + lane; b < u_hi; b += 32) own += bytes_of(b);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        pre += __shfl_xor_sync(FULL, pre, o);
-        own += __shfl_xor_sync(FULL, own, o);
-    }
+    const unsigned bpu = (unsigned)(DEC_U * 32) >> lgb;  // blocks per unit: 16 to 128
+    // width bytes, 16 at a time (the array is zero padded to 16; a unit and a
+    // tile start at multiples of 16)
+    const uint4* const w = (const uint4*)(it.cin + 32);
+    const unsigned v_end = (unsigned)(ceil16(nb) / 16);
+    const unsigned v_pre = min(t * NWARPS * bpu / 16, v_end);
+    unsigned pre = 0u;  // planes: at most 25 per block
+#pragma unroll 4
+    for (unsigned v = tid; v < v_pre; v += NTHREADS) pre += planes16(__ldg(w + v), nullptr, 0ull);
+    const unsigned v_lo = (t * NWARPS + warp) * (bpu / 16) + lane;
+    unsigned own = 0u;
+    if (lane < (int)(bpu / 16) && v_lo < v_end) own = planes16(__ldg(w + v_lo), nullptr, 0ull);
+    pre = __reduce_add_sync(FULL, pre);
+    own = __reduce_add_sync(FULL, own);
     if (lane == 0) {
         s_pre[warp] = pre;
         s_own[warp] = own;
     }
     __syncthreads();
-    unsigned long long off = 0ull, total = 0ull;
+    unsigned off = 0u, total = 0u;
 #pragma unroll
     for (int v = 0; v < NWARPS; ++v) {
-        off += s_pre[v] + (v < warp ? s_own[v] : 0ull);
+        off += s_pre[v] + (v < warp ? s_own[v] : 0u);
         total += s_pre[v] + s_own[v];
     }
-    if (t + 1 == it.ntiles && tid == 0 &&
-        total != __ldg((const unsigned long long*)it.cin + 3))
+    if (t + 1 == it.ntiles && tid == 0 && total * PB != __ldg((const unsigned long long*)it.cin + 3))
         fail(ctl, ZC_ERR_FORMAT, item_idx);
-    return off;
+    return off * PB;
 }
 
 // NWARPS warp units per CTA, one per warp, independent of each other; the
 // block size comes from the stream's header.
-// 5 CTAs per SM (48 registers): the decoder waits on its plane loads, and the
-// extra warps hide more of that than the few spilled values cost (measured on
-// the 512^3 field: 0.166 ms at 5 CTAs per SM, 0.175 ms at 4, 0.168 ms at 6)
-// BATCH: a multi-item launch (items may find their own unit offsets); the
-// single-stream decoder is compiled without that path, which would cost it
-// registers.
-template <bool BATCH>
+// BATCH: a multi-item launch; LOCAL: (some) items find their own unit offsets.
+// The decoder of a single scanned stream is compiled without that path, which
+// would cost it registers.
+template <bool BATCH, bool LOCAL>
 __device__ __forceinline__ void decompress_tile(const Launch& P)
 {
     extern __shared__ __align__(128) uint8_t dsm[];
@@ -1414,6 +1494,13 @@ __device__ __forceinline__ void decompress_tile(const Launch& P)
     }
     Item it = P.items != nullptr ? P.items[idx] : P.one;
     resolve_packed(P, it, idx);
+    // a workspace that is not initialised is refused (by the width scan where
+    // there is one; batched items of a few tiles never had one)
+    if (LOCAL && it.nchunks == 0 && (!BATCH || it.ntiles > DEC_LOCAL_TILES) &&
+        ld_volatile_u32(&P.ctl->magic) != WS_MAGIC) {
+        if (threadIdx.x == 0) fail(P.ctl, ZC_ERR_WORKSPACE, 0);
+        return;
+    }
     const unsigned t = tile - it.tile_begin;
     const int warp = threadIdx.x >> 5;
     const unsigned long long ue0 = ((unsigned long long)t * NWARPS + warp) * (DEC_U * 32);
@@ -1422,14 +1509,14 @@ __device__ __forceinline__ void decompress_tile(const Launch& P)
     float eb_in;
     const int lg = check_header(it, P.ctl, idx, -1, eb_in, threadIdx.x == 0 && t == 0);
     long long loff = -1;  // the unit's payload offset, when this CTA finds it
-    if (BATCH && it.nchunks == 0 && lg >= 4)  // uniform in the CTA
+    if (LOCAL && it.nchunks == 0 && lg >= 4)  // uniform in the CTA
         loff = (long long)local_unit_offset(it, lg, t, P.ctl, idx);
     // the width scan's offsets are read from here on: a single-stream decoder
     // launched dependent on the scan has looked up its tile and checked the
     // header while the scan ran, and waits for it now.  Every thread passes
     // this wait, so the decoder never completes before the scan (later
     // launches on the stream find the scan finished).
-    if (!BATCH) grid_dep_wait();
+    if (!BATCH && !LOCAL) grid_dep_wait();
     if (ue0 >= it.n) return;
     const float two = __fadd_rn(eb_in, eb_in);
     if (it.out_dtype == ZC_F32) {
@@ -1461,10 +1548,10 @@ __device__ __forceinline__ void decompress_tile(const Launch& P)
     else if (lg == -3) unit_raw_copy(it, ZC_BF16, ue0);
 }
 
-template <bool BATCH>
+template <bool BATCH, bool LOCAL>
 __global__ void __launch_bounds__(NTHREADS, DEC_CTAS_PER_SM) k_decompress(const Launch P)
 {
-    decompress_tile<BATCH>(P);
+    decompress_tile<BATCH, LOCAL>(P);
 }
 
 #endif  // ZC_DECODE_KERNELS

@@ -39,17 +39,20 @@ cudaError_t launch_group(Item* items, unsigned n_items, unsigned* part, unsigned
 
 cudaError_t launch_decompress(const Launch& P, unsigned grid, cudaStream_t s, bool after_wscan)
 {
-    const cudaError_t e1 = smem_limit<k_decompress<true>>(DEC_SMEM_BYTES);
-    const cudaError_t e0 = smem_limit<k_decompress<false>>(DEC_SMEM_BYTES);
-    if (e1 != cudaSuccess || e0 != cudaSuccess) return e1 != cudaSuccess ? e1 : e0;
     if (P.items != nullptr) {
-        k_decompress<true><<<grid, NTHREADS, DEC_SMEM_BYTES, s>>>(P);
+        const cudaError_t e = smem_limit<k_decompress<true, true>>(DEC_SMEM_BYTES);
+        if (e != cudaSuccess) return e;
+        k_decompress<true, true><<<grid, NTHREADS, DEC_SMEM_BYTES, s>>>(P);
         return cudaGetLastError();
     }
     if (!after_wscan) {
-        k_decompress<false><<<grid, NTHREADS, DEC_SMEM_BYTES, s>>>(P);
+        const cudaError_t e = smem_limit<k_decompress<false, true>>(DEC_SMEM_BYTES);
+        if (e != cudaSuccess) return e;
+        k_decompress<false, true><<<grid, NTHREADS, DEC_SMEM_BYTES, s>>>(P);
         return cudaGetLastError();
     }
+    const cudaError_t e = smem_limit<k_decompress<false, false>>(DEC_SMEM_BYTES);
+    if (e != cudaSuccess) return e;
     // launched dependent on the width scan just before it on the stream: its
     // CTAs read their headers and width bytes while the scan still runs
     cudaLaunchConfig_t cfg = {};
@@ -62,7 +65,7 @@ cudaError_t launch_decompress(const Launch& P, unsigned grid, cudaStream_t s, bo
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_decompress<false>, P);
+    return cudaLaunchKernelEx(&cfg, k_decompress<false, false>, P);
 }
 
 }  // namespace zc

@@ -45,6 +45,7 @@ cudaError_t launch_batch_u(const Launch& P, unsigned grid, cudaStream_t s);
 cudaError_t launch_wscan(const Launch& P, unsigned grid, cudaStream_t s);
 // after_wscan (single streams): the width scan was the launch just before on
 // `s`; the decoder is launched dependent on it (programmatic serialisation).
+// A single stream without one finds its offsets itself (nchunks 0).
 cudaError_t launch_decompress(const Launch& P, unsigned grid, cudaStream_t s,
                               bool after_wscan = false);
 // Item of every tile (by_chunk: of every width-scan chunk) of a multi-item
