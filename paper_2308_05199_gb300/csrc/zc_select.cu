@@ -81,22 +81,6 @@ __device__ __forceinline__ void load_span4(const Item& it, bool vec, unsigned lo
     }
 }
 
-// Largest block |delta| of the lane's block at blocks of G lanes (L = 4G):
-// the block's first lane contributes |q| of its first element (the head is
-// predicted from 0), every other lane |d| of its first element.
-// (xor shuffles within aligned groups of G lanes: every lane takes part with
-// the full mask, so no group waits for another)
-template <int G>
-__device__ __forceinline__ unsigned block_max(unsigned rest, unsigned e0q, unsigned e0d)
-{
-    const int lane = threadIdx.x & 31;
-    unsigned v = max(rest, (lane & (G - 1)) == 0 ? e0q : e0d);
-    if (G == 32) return __reduce_max_sync(FULL, v);
-#pragma unroll
-    for (int off = G / 2; off; off >>= 1) v = max(v, __shfl_xor_sync(FULL, v, off));
-    return v;
-}
-
 // One span of cnt elements (v: this lane's four); returns the span's L = 32
 // block bits (the same in every lane).  FULL: cnt == 128.  Branch-free:
 // elements outside the span, and the differences that do not exist at the
@@ -154,15 +138,29 @@ __device__ __forceinline__ unsigned stat_span(const float v[4], int cnt, const I
         A.nz_d += (v1 && d[m] == 0) ? 1u : 0u;
         if (m > 0) rest = max(rest, ad);
         A.sum_ad2 += ad2;
-        const bool sc = (d[m] > 0 && pd[m] < 0) || (d[m] < 0 && pd[m] > 0);
+        const bool sc = (d[m] ^ pd[m]) < 0 && d[m] != 0 && pd[m] != 0;
         A.n_sc += (v2 && sc) ? 1u : 0u;
     }
     const unsigned e0q = ok[0] ? (unsigned)abs(q[0]) : 0u;
     const unsigned e0d = (ok[0] && i0 >= 1) ? (unsigned)abs(d[0]) : 0u;
-    const unsigned m16 = block_max<4>(rest, e0q, e0d);
-    const unsigned m32 = block_max<8>(rest, e0q, e0d);
-    const unsigned m64 = block_max<16>(rest, e0q, e0d);
-    const unsigned m128 = block_max<32>(rest, e0q, e0d);
+    // Largest block |delta| at blocks of 4, 8, 16 and 32 lanes, right in each
+    // block's first lane: the block's first element counts as |q| (the head is
+    // predicted from 0), every other lane's first element as |d|.  A block of
+    // twice the size takes both halves and the second half's first |d|: five
+    // shuffles for the four sizes (ten when each size reduced by itself).
+    unsigned a = max(rest, (lane & 3) ? e0d : 0u);
+    a = max(a, __shfl_xor_sync(FULL_MASK_ALL, a, 1));
+    a = max(a, __shfl_xor_sync(FULL_MASK_ALL, a, 2));
+    const unsigned m16 = max(a, e0q);
+    if ((lane & 7) == 4) a = max(a, e0d);
+    a = max(a, __shfl_xor_sync(FULL_MASK_ALL, a, 4));
+    const unsigned m32 = max(a, e0q);
+    if ((lane & 15) == 8) a = max(a, e0d);
+    a = max(a, __shfl_xor_sync(FULL_MASK_ALL, a, 8));
+    const unsigned m64 = max(a, e0q);
+    if (lane == 16) a = max(a, e0d);
+    a = max(a, __shfl_xor_sync(FULL_MASK_ALL, a, 16));
+    const unsigned m128 = max(a, e0q);
     const unsigned b32 = ((lane & 7) == 0 && m32) ? (bitlen_u(m32) + 1) * 32 : 0u;
     A.b16 += ((lane & 3) == 0 && m16) ? (bitlen_u(m16) + 1) * 16 : 0u;
     A.b64 += ((lane & 15) == 0 && m64) ? (bitlen_u(m64) + 1) * 64 : 0u;
