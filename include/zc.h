@@ -418,6 +418,17 @@ int zc_mlp_grad(const float* d_params, const float* d_norm, const float* d_x, co
 int zc_mlp_sgd(float* d_params, float* d_vel, const float* d_grad, float lr, float momentum,
                zc_stream_t s);
 
+/* One epoch of minibatch momentum SGD over the N rows d_idx[0 .. N) of d_x /
+ * d_t, `batch` rows at a time (the last minibatch takes what is left): for
+ * each minibatch the gradient, then the update, as zc_mlp_grad and zc_mlp_sgd
+ * define them, sums in a fixed order.  d_grad receives the last minibatch's
+ * gradient, d_losses[ceil(N / batch)] every minibatch's loss.  Scratch as for
+ * zc_mlp_grad of `batch` rows (large minibatches use it). */
+int zc_mlp_fit_epoch(float* d_params, float* d_vel, float* d_grad, const float* d_norm,
+                     const float* d_x, const float* d_t, const int* d_idx, int N, int batch,
+                     double lr, double momentum, float* d_losses, void* d_scratch,
+                     size_t scratch_bytes, zc_stream_t s);
+
 /* Cost model of the selection: a message of n elements of s bytes costs,
  * coded at L_k with b bits per element, n s ns_per_byte[k] + (n b / 8) /
  * link_gbs ns, and raw, n s raw_ns_per_byte + (32 + n s) / link_gbs ns

@@ -6,6 +6,7 @@
 // comment of zc.h (zc_batch_chunk_stats .. zc_batch_select).  Everything runs
 // on the device; nothing is read back, so a whole select-then-compress
 // sequence can be captured in one CUDA graph.
+#include <cooperative_groups.h>
 #include <cstddef>
 #include <cstring>
 
@@ -566,6 +567,383 @@ __global__ void k_mlp_sgd(float* P, float* V, const float* G, float lr, float mo
     P[p] = __fsub_rn(P[p], __fmul_rn(lr, v));
 }
 
+// ---- a training epoch in one launch ------------------------------------------------
+// A minibatch is a chain of three small launches (gradient of one CTA per 64
+// rows, reduction, update), each of which loads the parameters anew; at 256
+// rows it keeps 4 SMs busy, and an epoch of 10000 rows took 1545 us.  Here one
+// cluster of FC CTAs trains for the whole epoch with the parameters in the
+// shared memory of every CTA (359 us; with the permutation and the
+// host's part of the epoch 573 us).  It does the very same
+// arithmetic in the same order, so an epoch's results are those of the chain,
+// bit for bit: a ReLU whose input is a rounding away from 0 would otherwise
+// take the other side in one of the two.
+//
+// A turn takes 4 tiles of TB rows (the chain's CTAs).  Tile g is worked on by
+// the CTAs 4 g .. 4 g + 3 ("quarters"):
+//   rows: each quarter runs 16 of the tile's rows forward and backward and
+//     writes their activations and deltas to the quarters that need them
+//     (distributed shared memory);
+//   sums: each quarter sums its share of the tile's gradient over all 64 rows
+//     in order: the neurons j of both hidden layers with j / 16 = quarter, and
+//     output o = quarter;
+//   totals: a quarter's four CTAs (one per tile) add a quarter of its share
+//     each over the tiles, in order; after the minibatch's last turn they
+//     update velocity and parameters and write these into every CTA's copy.
+// A cluster barrier closes every phase.
+// What bounds it is the instructions of a warp's share, a serial chain of
+// phases (256 threads per CTA: 3500 instructions per warp and minibatch of 256,
+// 15.5 us; the sums over rows cannot be split further without another order).
+constexpr int FC = 16, FT = 4;       // CTAs, tiles per turn
+constexpr int FM = 512;              // threads per CTA
+constexpr int FQ = FC / FT;          // quarters of a tile
+constexpr int FR = TB / FQ;          // rows of a quarter
+constexpr int FJ = NH / FQ;          // neurons of a quarter
+// Larger minibatches keep more SMs busy in the chain than one cluster has:
+// measured
+// per epoch, cluster / chain: 10000 rows by 64 1349 / 5153 us, by 256 359 / 1318, by
+// 1000 302 / 343; 16384 rows by 2048 460 / 267.
+constexpr int FIT_MAX_BATCH = 1024;
+// Shared-memory rows are padded so that 16-byte accesses of consecutive rows
+// fall in distinct banks.
+struct FitNet {
+    alignas(16) float W1[NH][NIP];
+    alignas(16) float W2[NH][NHP];
+    alignas(16) float W3[NO][NHP];
+    float b1[NH], b2[NH], b3[NO];
+};
+// A quarter's share of a tile's gradient, FSHARE floats: W2 rows, W1 rows, the
+// W3 row, then the biases b2, b1, b3 and the sum of squares (quarter 0's).
+constexpr int QS_W1 = FJ * NH, QS_W3 = QS_W1 + FJ * NI, QS_B2 = QS_W3 + NH, QS_B1 = QS_B2 + FJ,
+              QS_B3 = QS_B1 + FJ, QS_LOSS = QS_B3 + 1, FSHARE = QS_LOSS + 1;
+constexpr int FOWN = (FSHARE + FT - 1) / FT;  // of it, per CTA of the quarter
+static_assert(FOWN <= FM && FQ == NO && NH % FQ == 0, "one entry per thread");
+struct FitSmem {
+    FitNet net;
+    alignas(16) float X[2][TB][NIP];
+    float T[2][FR][NO];
+    alignas(16) float A1[TB][NHP];   // activations of the tile's rows
+    alignas(16) float A2[TB][NHP];
+    float D2q[TB][FJ + 1];           // dA2 and dA1 of the quarter's neurons
+    float D1q[TB][FJ + 1];
+    float Yq[TB];                    // dY of the quarter's output
+    alignas(16) float D2[FR][NHP];   // dA2 of this CTA's rows
+    float Y[FR][NO];                 // their dY
+    float red[2 * FQ];               // squares of eight rows each (in quarter 0)
+    alignas(16) float G[FSHARE];
+};
+
+// Parameter of entry e of quarter q's share (NPARAM: the loss, -1: none).
+__device__ __forceinline__ int fit_param(int q, int e)
+{
+    if (e < QS_W1) return OFF_W2 + q * FJ * NH + e;
+    if (e < QS_W3) return q * FJ * NI + (e - QS_W1);
+    if (e < QS_B2) return OFF_W3 + q * NH + (e - QS_W3);
+    if (e < QS_B1) return OFF_B2 + q * FJ + (e - QS_B2);
+    if (e < QS_B3) return OFF_B1 + q * FJ + (e - QS_B1);
+    if (e < QS_LOSS) return OFF_B3 + q;
+    return e == QS_LOSS && q == 0 ? NPARAM : -1;
+}
+__device__ __forceinline__ float* fit_slot(FitNet& n, int p)
+{
+    if (p < OFF_B1) return &n.W1[p / NI][p % NI];
+    if (p < OFF_W2) return &n.b1[p - OFF_B1];
+    if (p < OFF_B2) return &n.W2[(p - OFF_W2) / NH][(p - OFF_W2) % NH];
+    if (p < OFF_W3) return &n.b2[p - OFF_B2];
+    if (p < OFF_B3) return &n.W3[(p - OFF_W3) / NH][(p - OFF_W3) % NH];
+    return &n.b3[p - OFF_B3];
+}
+
+// Shared-memory address `a` in CTA `rank` of the cluster, and access to it.
+__device__ __forceinline__ unsigned peer_addr(const void* a, unsigned rank)
+{
+    unsigned r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(a)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void peer_store(unsigned a, float v)
+{
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ float peer_load(unsigned a)
+{
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// This CTA's rows (`rows` of them real) of the tile in sm.X[buf]; quarter q of
+// the tile is CTA rank0 + q.
+__device__ __forceinline__ void fit_rows(FitSmem& sm, unsigned rank0, int quarter, int buf, int rows,
+                                         float scale)
+{
+    const int t = threadIdx.x, j = t & (NH - 1);
+    constexpr int RT = FR / (FM / NH);         // rows per thread
+    const int s0 = (t / NH) * RT, r0 = quarter * FR;  // first row here, first row in the tile
+    FitNet& n = sm.net;
+    {
+        float acc[RT];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) acc[i] = n.b1[j];
+#pragma unroll
+        for (int k = 0; k < NI; k += 4) {
+            const float4 w = *reinterpret_cast<const float4*>(&n.W1[j][k]);
+#pragma unroll
+            for (int i = 0; i < RT; ++i) {
+                const float4 x = *reinterpret_cast<const float4*>(&sm.X[buf][r0 + s0 + i][k]);
+                acc[i] = __fmaf_rn(w.x, x.x, acc[i]);
+                acc[i] = __fmaf_rn(w.y, x.y, acc[i]);
+                acc[i] = __fmaf_rn(w.z, x.z, acc[i]);
+                acc[i] = __fmaf_rn(w.w, x.w, acc[i]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < FQ; ++q) {
+            const unsigned a = peer_addr(&sm.A1[r0 + s0][j], rank0 + q);
+#pragma unroll
+            for (int i = 0; i < RT; ++i) peer_store(a + i * (int)sizeof(sm.A1[0]), relu(acc[i]));
+        }
+    }
+    __syncthreads();
+    {
+        float acc[RT];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) acc[i] = n.b2[j];
+#pragma unroll 4
+        for (int k = 0; k < NH; k += 4) {
+            const float4 w = *reinterpret_cast<const float4*>(&n.W2[j][k]);
+#pragma unroll
+            for (int i = 0; i < RT; ++i) {
+                const float4 a = *reinterpret_cast<const float4*>(&sm.A1[r0 + s0 + i][k]);
+                acc[i] = __fmaf_rn(w.x, a.x, acc[i]);
+                acc[i] = __fmaf_rn(w.y, a.y, acc[i]);
+                acc[i] = __fmaf_rn(w.z, a.z, acc[i]);
+                acc[i] = __fmaf_rn(w.w, a.w, acc[i]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < FQ; ++q) {
+            const unsigned a = peer_addr(&sm.A2[r0 + s0][j], rank0 + q);
+#pragma unroll
+            for (int i = 0; i < RT; ++i) peer_store(a + i * (int)sizeof(sm.A2[0]), relu(acc[i]));
+        }
+    }
+    __syncthreads();
+    if (t < FR * NO) {  // outputs, their deltas and the squares of eight rows per warp
+        const int s = t / NO, o = t % NO;
+        float y = n.b3[o];
+#pragma unroll 4
+        for (int k = 0; k < NH; k += 4) {
+            const float4 w = *reinterpret_cast<const float4*>(&n.W3[o][k]);
+            const float4 a = *reinterpret_cast<const float4*>(&sm.A2[r0 + s][k]);
+            y = __fmaf_rn(w.x, a.x, y);
+            y = __fmaf_rn(w.y, a.y, y);
+            y = __fmaf_rn(w.z, a.z, y);
+            y = __fmaf_rn(w.w, a.w, y);
+        }
+        float sq = 0.0f, dy = 0.0f;
+        if (s < rows) {
+            const float res = __fsub_rn(y, sm.T[buf][s][o]);
+            sq = __fmul_rn(res, res);
+            dy = __fmul_rn(scale, res);
+        }
+        sm.Y[s][o] = dy;
+        peer_store(peer_addr(&sm.Yq[r0 + s], rank0 + o), dy);
+#pragma unroll
+        for (int off = 16; off; off >>= 1) sq = __fadd_rn(sq, __shfl_xor_sync(FULL, sq, off));
+        if ((t & 31) == 0) peer_store(peer_addr(&sm.red[2 * quarter + (t >> 5)], rank0), sq);
+    }
+    __syncthreads();
+    const unsigned d2 = peer_addr(&sm.D2q[r0 + s0][j % FJ], rank0 + j / FJ);
+#pragma unroll
+    for (int i = 0; i < RT; ++i) {  // dA2[s][j] = (sum_o dY[s][o] W3[o][j]) [H2 > 0]
+        const int s = s0 + i;
+        float a = 0.0f;
+#pragma unroll
+        for (int o = 0; o < NO; ++o) a = __fadd_rn(a, __fmul_rn(sm.Y[s][o], n.W3[o][j]));
+        const float d = sm.A2[r0 + s][j] > 0.0f ? a : 0.0f;
+        sm.D2[s][j] = d;
+        peer_store(d2 + i * (int)sizeof(sm.D2q[0]), d);
+    }
+    __syncthreads();
+    {  // dA1[s][k] = (sum_j dA2[s][j] W2[j][k]) [H1 > 0] (k = this thread's j)
+        float acc[RT];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) acc[i] = 0.0f;
+#pragma unroll 4
+        for (int jj = 0; jj < NH; jj += 4) {
+            const float w0 = n.W2[jj][j], w1 = n.W2[jj + 1][j], w2 = n.W2[jj + 2][j], w3 = n.W2[jj + 3][j];
+#pragma unroll
+            for (int i = 0; i < RT; ++i) {
+                const float4 d = *reinterpret_cast<const float4*>(&sm.D2[s0 + i][jj]);
+                acc[i] = __fadd_rn(acc[i], __fmul_rn(d.x, w0));
+                acc[i] = __fadd_rn(acc[i], __fmul_rn(d.y, w1));
+                acc[i] = __fadd_rn(acc[i], __fmul_rn(d.z, w2));
+                acc[i] = __fadd_rn(acc[i], __fmul_rn(d.w, w3));
+            }
+        }
+        const unsigned d1 = peer_addr(&sm.D1q[r0 + s0][j % FJ], rank0 + j / FJ);
+#pragma unroll
+        for (int i = 0; i < RT; ++i)
+            peer_store(d1 + i * (int)sizeof(sm.D1q[0]), sm.A1[r0 + s0 + i][j] > 0.0f ? acc[i] : 0.0f);
+    }
+}
+
+// This quarter's share of the tile's gradient, rows in order.
+__device__ __forceinline__ void fit_sums(FitSmem& sm, int quarter, int buf)
+{
+    const int t = threadIdx.x;
+    constexpr int HT = FM / 2;
+    const int u = t % HT, j = u >> 4, k = u & 15;
+    static_assert(HT == FJ * 16 && NI == 16 && NH == 64, "thread mapping");
+    if (t < HT) {  // W2: neuron j, inputs 4 k .. 4 k + 3
+        float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
+#pragma unroll 8
+        for (int s = 0; s < TB; ++s) {
+            const float d2 = sm.D2q[s][j];
+            const float4 a = *reinterpret_cast<const float4*>(&sm.A1[s][4 * k]);
+            a0 = __fadd_rn(a0, __fmul_rn(d2, a.x));
+            a1 = __fadd_rn(a1, __fmul_rn(d2, a.y));
+            a2 = __fadd_rn(a2, __fmul_rn(d2, a.z));
+            a3 = __fadd_rn(a3, __fmul_rn(d2, a.w));
+        }
+        *reinterpret_cast<float4*>(&sm.G[j * NH + 4 * k]) = make_float4(a0, a1, a2, a3);
+        return;
+    }
+    // W1: neuron j, input k; some threads one more sum: the W3 row, then the
+    // biases b2, b1, b3 (which follow one another in the share)
+    float w1 = 0.0f, e = 0.0f;
+#pragma unroll 8
+    for (int s = 0; s < TB; ++s) w1 = __fadd_rn(w1, __fmul_rn(sm.D1q[s][j], sm.X[buf][s][k]));
+    sm.G[QS_W1 + j * NI + k] = w1;
+    if (u < NH) {
+#pragma unroll 8
+        for (int s = 0; s < TB; ++s) e = __fadd_rn(e, __fmul_rn(sm.Yq[s], sm.A2[s][u]));
+    } else if (u < NH + 2 * FJ + 1) {
+        const int b = u - NH;  // a column of D2q, of D1q, or Yq
+        const float* const src = b < FJ ? &sm.D2q[0][b] : b < 2 * FJ ? &sm.D1q[0][b - FJ] : sm.Yq;
+        const int stride = b < 2 * FJ ? FJ + 1 : 1;
+#pragma unroll 8
+        for (int s = 0; s < TB; ++s) e = __fadd_rn(e, src[s * stride]);
+    } else if (u == HT - 1 && quarter == 0) {
+#pragma unroll
+        for (int w = 0; w < 2 * FQ; ++w) e = __fadd_rn(e, sm.red[w]);
+    }
+    if (u < NH + 2 * FJ + 1) sm.G[QS_W3 + u] = e;
+    else if (u == HT - 1) sm.G[QS_LOSS] = e;
+}
+
+__global__ void __launch_bounds__(FM, 1) k_mlp_fit(float* P, float* V, float* grad, const float* norm,
+                                                const float* X, const float* T, const int* idx,
+                                                int N, int batch, float lr, float momentum,
+                                                float* losses)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    extern __shared__ __align__(16) uint8_t raw[];
+    FitSmem& sm = *reinterpret_cast<FitSmem*>(raw);
+    const int t = threadIdx.x, c = (int)cluster.block_rank();
+    const int tile = c / FQ, quarter = c % FQ;
+    for (int p = t; p < NPARAM; p += FM) *fit_slot(sm.net, p) = P[p];
+    // this thread's entry of the quarter's share, its parameter and its place
+    const int ent = t < FOWN && tile * FOWN + t < FSHARE ? tile * FOWN + t : -1;
+    const int par = ent >= 0 ? fit_param(quarter, ent) : -1;
+    const bool trained = par >= 0 && par < NPARAM;
+    float pv = trained ? P[par] : 0.0f, vv = trained ? V[par] : 0.0f;
+    const float* const slot = trained ? fit_slot(sm.net, par) : nullptr;
+    const int k = t % NI, xr = t / NI;  // input of this thread, its rows xr + 16 i of the tile
+    constexpr int XI = TB * NI / FM;
+    static_assert(FM % NI == 0 && NO * FR <= FM, "input elements per thread");
+    const int ts = t / NO, to = t % NO;  // target of the threads below FR * NO
+    const bool has_t = t < FR * NO;
+    const float nm = norm[k], ni = norm[NI + k];
+    const int steps = (N + batch - 1) / batch;
+    // Row r of this CTA's tile in turn q of minibatch m: its place in idx, or -1.
+    auto place = [&](int m, int q, int r) {
+        if (m >= steps) return -1;
+        const int b = (q * FT + tile) * TB + r;
+        return b < min(batch, N - m * batch) ? m * batch + b : -1;
+    };
+    auto next = [&](int& m, int& q) {
+        if (m < steps && ++q * FT * TB >= min(batch, N - m * batch)) {
+            q = 0;
+            ++m;
+        }
+    };
+    // Inputs are fetched a turn ahead, their row numbers two turns ahead.
+    int rx[XI], rt;
+    auto fetch_rows = [&](int m, int q) {
+#pragma unroll
+        for (int i = 0; i < XI; ++i) {
+            const int at = place(m, q, xr + (FM / NI) * i);
+            rx[i] = at >= 0 ? idx[at] : -1;
+        }
+        const int at = has_t ? place(m, q, quarter * FR + ts) : -1;
+        rt = at >= 0 ? idx[at] : -1;
+    };
+    float xv[XI], tv;
+    auto fetch = [&] {
+#pragma unroll
+        for (int i = 0; i < XI; ++i)
+            xv[i] = rx[i] >= 0 ? X[(long long)rx[i] * NI + k] : nm;  // (normalises to 0)
+        tv = rt >= 0 ? T[(long long)rt * NO + to] : 0.0f;
+    };
+    auto put = [&](int buf) {
+#pragma unroll
+        for (int i = 0; i < XI; ++i)  // normalised here, when the loads have long arrived
+            sm.X[buf][xr + (FM / NI) * i][k] = __fmul_rn(__fsub_rn(xv[i], nm), ni);
+        if (has_t) sm.T[buf][ts][to] = tv;
+    };
+    int m2 = 0, q2 = 0;  // the turn whose row numbers are fetched next
+    fetch_rows(m2, q2);
+    next(m2, q2);
+    fetch();
+    put(0);
+    fetch_rows(m2, q2);
+    next(m2, q2);
+    int buf = 0;
+    cluster.sync();
+    for (int m = 0; m < steps; ++m) {
+        const int B = min(batch, N - m * batch);
+        const float scale = 2.0f / (float)(B * NO);
+        float acc = 0.0f;
+        for (int b0 = 0; b0 < B; b0 += FT * TB, buf ^= 1) {
+            fetch();
+            fetch_rows(m2, q2);
+            next(m2, q2);
+            const int tiles = min(FT, (B - b0 + TB - 1) / TB);  // of this turn
+            if (tile < tiles)
+                fit_rows(sm, tile * FQ, quarter, buf, min(FR, max(0, B - b0 - tile * TB - quarter * FR)), scale);
+            put(buf ^ 1);
+            cluster.sync();  // the tiles' rows are complete
+            if (tile < tiles) fit_sums(sm, quarter, buf);
+            cluster.sync();  // the tiles' sums are complete, nobody reads the parameters
+            if (ent >= 0) {
+                float g[FT];
+#pragma unroll
+                for (int r = 0; r < FT; ++r)
+                    if (r < tiles) g[r] = peer_load(peer_addr(&sm.G[ent], r * FQ + quarter));
+#pragma unroll
+                for (int r = 0; r < FT; ++r)
+                    if (r < tiles) acc = __fadd_rn(acc, g[r]);
+            }
+        }
+        if (trained) {
+            vv = __fadd_rn(__fmul_rn(momentum, vv), acc);
+            pv = __fsub_rn(pv, __fmul_rn(lr, vv));
+#pragma unroll
+            for (int r = 0; r < FC; ++r) peer_store(peer_addr(slot, r), pv);
+            if (m + 1 == steps) {
+                P[par] = pv;
+                V[par] = vv;
+                grad[par] = acc;
+            }
+        } else if (par == NPARAM) {
+            losses[m] = acc / (float)(B * NO);
+        }
+        cluster.sync();
+    }
+}
+
 // ---- selection: one thread per item -------------------------------------------------
 struct SelectArgs {
     float link, c[4], c_raw, judge, judge_time;
@@ -702,6 +1080,51 @@ int zc_mlp_sgd(float* d_params, float* d_vel, const float* d_grad, float lr, flo
     k_mlp_sgd<<<(NPARAM + 255) / 256, 256, 0, (cudaStream_t)s>>>(d_params, d_vel, d_grad, lr,
                                                                  momentum);
     return cudaGetLastError() == cudaSuccess ? ZC_OK : ZC_ERR_CUDA;
+}
+
+int zc_mlp_fit_epoch(float* d_params, float* d_vel, float* d_grad, const float* d_norm,
+                     const float* d_x, const float* d_t, const int* d_idx, int N, int batch,
+                     double lr, double momentum, float* d_losses, void* d_scratch,
+                     size_t scratch_bytes, zc_stream_t s)
+{
+    if (N < 0 || batch < 1) return ZC_ERR_ARG;
+    if (N == 0) return ZC_OK;
+    if (d_params == nullptr || d_vel == nullptr || d_grad == nullptr || d_norm == nullptr ||
+        d_x == nullptr || d_t == nullptr || d_idx == nullptr || d_losses == nullptr)
+        return ZC_ERR_ARG;
+    if (batch > N) batch = N;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(FC);
+    cfg.blockDim = dim3(FM);
+    cfg.dynamicSmemBytes = sizeof(FitSmem);
+    cfg.stream = (cudaStream_t)s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = FC;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    // (a partition of the GPU may have no room for a cluster of this size)
+    int clusters = 0;
+    bool fits = batch <= FIT_MAX_BATCH && smem_limit<k_mlp_fit>((int)sizeof(FitSmem)) == cudaSuccess &&
+                cudaFuncSetAttribute(k_mlp_fit, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                cudaOccupancyMaxActiveClusters(&clusters, k_mlp_fit, &cfg) == cudaSuccess && clusters > 0;
+    if (!fits) {
+        cudaGetLastError();
+        for (int m = 0; (long long)m * batch < N; ++m) {
+            const int B = N - m * batch < batch ? N - m * batch : batch;
+            int st = zc_mlp_grad(d_params, d_norm, d_x, d_t, d_idx + (size_t)m * batch, B, d_grad,
+                                 d_losses + m, d_scratch, scratch_bytes, s);
+            if (st == ZC_OK) st = zc_mlp_sgd(d_params, d_vel, d_grad, (float)lr, (float)momentum, s);
+            if (st != ZC_OK) return st;
+        }
+        return ZC_OK;
+    }
+    return cudaLaunchKernelEx(&cfg, k_mlp_fit, d_params, d_vel, d_grad, d_norm, d_x, d_t, d_idx, N,
+                              batch, (float)lr, (float)momentum, d_losses) == cudaSuccess
+               ? ZC_OK
+               : ZC_ERR_CUDA;
 }
 
 int zc_batch_select_timed(const zc_batch* plan, const float* d_feat, const float* d_pred,

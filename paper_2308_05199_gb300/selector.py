@@ -380,17 +380,12 @@ class Mlp:
         hist = []
         for _ in range(epochs):
             with torch.cuda.stream(ts):
-                idx.copy_(torch.randperm(N, generator=g, device=X.device).to(torch.int32))
-            for k in range(steps):
-                b0 = k * batch
-                B = min(batch, N - b0)
-                zc._check(zc.zc_mlp_grad(self.params.data_ptr(), self.norm.data_ptr(),
-                                         X.data_ptr(), T.data_ptr(), idx.data_ptr() + 4 * b0, B,
-                                         self.grad.data_ptr(), losses.data_ptr() + 4 * k,
-                                         scratch.data_ptr(), scratch.numel() * 4, s),
-                          "zc_mlp_grad")
-                zc._check(zc.zc_mlp_sgd(self.params.data_ptr(), self.vel.data_ptr(),
-                                        self.grad.data_ptr(), lr, momentum, s), "zc_mlp_sgd")
+                idx.copy_(torch.randperm(N, generator=g, device=X.device))
+            zc._check(zc.zc_mlp_fit_epoch(self.params.data_ptr(), self.vel.data_ptr(),
+                                          self.grad.data_ptr(), self.norm.data_ptr(),
+                                          X.data_ptr(), T.data_ptr(), idx.data_ptr(), N, batch,
+                                          lr, momentum, losses.data_ptr(), scratch.data_ptr(),
+                                          scratch.numel() * 4, s), "zc_mlp_fit_epoch")
             with torch.cuda.stream(ts):
                 m = losses.mean()
             ts.synchronize()

@@ -144,6 +144,8 @@ def _declare(L):
         "zc_mlp_scratch_bytes": (sz, [i32]),
         "zc_mlp_grad": (i32, [vp, vp, vp, vp, vp, i32, vp, vp, vp, sz, vp]),
         "zc_mlp_sgd": (i32, [vp, vp, vp, c.c_float, c.c_float, vp]),
+        "zc_mlp_fit_epoch": (i32, [vp, vp, vp, vp, vp, vp, vp, i32, i32, c.c_double, c.c_double,
+                                   vp, vp, sz, vp]),
         "zc_batch_select": (i32, [c.POINTER(ZcBatch), vp, vp, c.POINTER(ZcSelectCfg), vp, vp,
                                   vp]),
         "zc_batch_select_timed": (i32, [c.POINTER(ZcBatch), vp, vp, vp, c.POINTER(ZcSelectCfg),
@@ -174,7 +176,7 @@ def exported_names():
             "zc_plan_compress_batch", "zc_compress_batch", "zc_plan_decompress_batch",
             "zc_decompress_batch", "zc_batch_set_grouped", "zc_plan_decompress_streams",
             "zc_autotune_batch", "zc_batch_chunk_stats", "zc_mlp_forward",
-            "zc_mlp_scratch_bytes", "zc_mlp_grad", "zc_mlp_sgd", "zc_batch_select",
+            "zc_mlp_scratch_bytes", "zc_mlp_grad", "zc_mlp_sgd", "zc_mlp_fit_epoch", "zc_batch_select",
             "zc_batch_select_timed",
             "zc_graph_begin", "zc_graph_end",
             "zc_graph_launch", "zc_graph_destroy",
@@ -346,6 +348,12 @@ def zc_mlp_grad(d_params, d_norm, d_x, d_t, d_idx, B, d_grad, d_loss, d_scratch,
 
 def zc_mlp_sgd(d_params, d_vel, d_grad, lr, momentum, stream) -> int:
     return lib().zc_mlp_sgd(d_params, d_vel, d_grad, lr, momentum, stream)
+
+
+def zc_mlp_fit_epoch(d_params, d_vel, d_grad, d_norm, d_x, d_t, d_idx, N, batch, lr, momentum,
+                     d_losses, d_scratch, scratch_bytes, stream) -> int:
+    return lib().zc_mlp_fit_epoch(d_params, d_vel, d_grad, d_norm, d_x, d_t, d_idx, N, batch, lr,
+                                  momentum, d_losses, d_scratch, scratch_bytes, stream)
 
 
 def zc_batch_select(plan, d_feat, d_pred, cfg, d_choice, d_counts, stream) -> int:
