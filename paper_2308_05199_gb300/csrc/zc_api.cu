@@ -140,7 +140,8 @@ int ws_view(void* ws, size_t bytes, WsView& v)
 // Width scans over at least this many items find a chunk's item in a map
 // (one extra launch); fewer items are searched (at most 8 dependent loads).
 constexpr int CHUNK_MAP_ITEMS = 256;
-// The fused step finds a tile's item by search up to this many items.
+// The fused step finds a tile's item by search up to this many items, in
+// launches of few tiles.
 constexpr int SEARCH_ITEMS = 16;
 
 // SM count of the current device (queried once per device).
@@ -262,13 +263,21 @@ cudaError_t launch_batch(int C, const Launch& P, unsigned grid, cudaStream_t s)
 
 inline uint64_t elem_bytes(int dtype) { return dtype == ZC_F32 ? 4 : 2; }
 
-// Largest item (in decode tiles) of a batched decompression that goes without
-// width-scan chunks.
-unsigned dec_local_tiles(int n_msgs, const zc_message* msgs)
+// Decompressions of at least this many elements take large units.
+constexpr uint64_t DEC_LARGE_N = 1ull << 26;
+
+// Units of a batched decompression (rows) and its largest item (in decode
+// tiles) that goes without width-scan chunks.
+int dec_units(int n_msgs, const zc_message* msgs, unsigned* local)
 {
-    uint64_t tiles = 0;
-    for (int i = 0; i < n_msgs; ++i) tiles += tiles_for(msgs[i].n, DEC_U);
-    return tiles <= LOCAL_LAUNCH_TILES ? DEC_LOCAL_FEW_TILES : DEC_LOCAL_TILES;
+    uint64_t tiles = 0, n = 0;
+    for (int i = 0; i < n_msgs; ++i) {
+        tiles += tiles_for(msgs[i].n, DEC_U);
+        n += msgs[i].n;
+    }
+    *local = tiles <= LOCAL_LAUNCH_TILES ? DEC_LOCAL_FEW_TILES : DEC_LOCAL_TILES;
+    // (items of less than a large tile would leave its warps without work)
+    return n >= DEC_LARGE_N && n / (uint64_t)n_msgs >= (uint64_t)NWARPS * DEC_U_LARGE * 32 * 4 ? DEC_U_LARGE : DEC_U;
 }
 
 }  // namespace
@@ -445,8 +454,9 @@ int zc_decompress(const void* d_cmp, size_t cmp_cap, void* d_out, uint64_t n, in
     WsView w;
     int st = ws_view(d_ws, ws_bytes, w);
     if (st) return st;
-    const uint64_t tiles = tiles_for(n, DEC_U);
-    const uint64_t chunks = tiles <= DEC_LOCAL_SINGLE_TILES ? 0 : chunks_for(tiles);
+    const int du = n >= DEC_LARGE_N ? DEC_U_LARGE : DEC_U;
+    const uint64_t tiles = tiles_for(n, du);
+    const uint64_t chunks = du == DEC_U && tiles <= DEC_LOCAL_SINGLE_TILES ? 0 : chunks_for(tiles);
     if (tiles * NWARPS > w.cap || tiles > 0x7fffffffull) return ZC_ERR_WORKSPACE;
     Launch P = base_launch(w);
     Item& it = P.one;
@@ -458,7 +468,7 @@ int zc_decompress(const void* d_cmp, size_t cmp_cap, void* d_out, uint64_t n, in
     it.nchunks = (unsigned)chunks;
     it.out_dtype = out_dtype;
     P.n_items = 1;
-    P.urows = DEC_U;
+    P.urows = du;
     P.total_tiles = (unsigned)chunks;
     if (chunks > 0 && launch_wscan(P, (unsigned)chunks, (cudaStream_t)s) != cudaSuccess) return ZC_ERR_CUDA;
     P.total_tiles = (unsigned)tiles;
@@ -620,10 +630,11 @@ int zc_reduce_step_batch(const zc_plan* plan, void* d_ws, size_t ws_bytes, zc_st
     // map is built while the width scan runs, the fused kernel's CTAs become
     // resident while the map finishes (both wait for their inputs).  Few
     // items are searched instead: one thread's few loads per tile, from L1
-    // after its CTA's first tile, against a launch of about 4 us
-    // (the five-rank recursive
-    // doubling of 1M elements: 142 us with maps, 139 us without).
-    if (plan->n_items > SEARCH_ITEMS) {
+    // after its CTA's first tile, against a launch of about 4 us (the
+    // five-rank recursive doubling of 1M elements: 142 us with maps, 139
+    // without).  Over many tiles the map is the faster one (8-rank ring of
+    // 8192^2: 1685 us with maps, 1710 without).
+    if (plan->n_items > (plan->total_tiles <= LOCAL_LAUNCH_TILES ? SEARCH_ITEMS : 1)) {
         if (launch_tile_map(P.items, P.n_items, P.total_tiles, w.tile_map, (cudaStream_t)s,
                             false, scan) != cudaSuccess)
             return ZC_ERR_CUDA;
@@ -848,7 +859,8 @@ int zc_plan_decompress_batch(zc_batch* plan, int n_msgs, const zc_message* h_msg
         return ZC_ERR_ARG;
     std::vector<Item> items((size_t)n_msgs);
     uint64_t tile = 0, chunk = 0;
-    const unsigned local = dec_local_tiles(n_msgs, h_msgs);
+    unsigned local;
+    const int du = dec_units(n_msgs, h_msgs, &local);
     for (int i = 0; i < n_msgs; ++i) {
         const zc_message& m = h_msgs[i];
         if (!dtype_ok(m.dtype) || (m.n > 0 && m.out == nullptr) ||
@@ -860,7 +872,7 @@ int zc_plan_decompress_batch(zc_batch* plan, int n_msgs, const zc_message* h_msg
         it.raw_out = m.out;
         it.n = m.n;
         it.tile_begin = (unsigned)tile;
-        it.ntiles = (unsigned)tiles_for(m.n, DEC_U);
+        it.ntiles = (unsigned)tiles_for(m.n, du);
         it.chunk_begin = (unsigned)chunk;
         it.nchunks = it.ntiles <= local ? 0u : (unsigned)chunks_for(it.ntiles);
         it.x_dtype = m.dtype;
@@ -874,7 +886,7 @@ int zc_plan_decompress_batch(zc_batch* plan, int n_msgs, const zc_message* h_msg
         return ZC_ERR_CUDA;
     std::memset(plan, 0, sizeof(*plan));
     plan->n_msgs = n_msgs;
-    plan->tile_chunks = 0;
+    plan->tile_chunks = du / 8;
     plan->grid = 0;
     plan->decompress = 1;
     plan->total_tiles = tile;
@@ -896,7 +908,8 @@ int zc_plan_decompress_streams(zc_batch* plan, int n_msgs, const void* const* h_
         return ZC_ERR_ARG;
     std::vector<Item> items((size_t)n_msgs);
     uint64_t tile = 0, chunk = 0;
-    const unsigned local = dec_local_tiles(n_msgs, h_msgs);
+    unsigned local;
+    const int du = dec_units(n_msgs, h_msgs, &local);
     for (int i = 0; i < n_msgs; ++i) {
         const zc_message& m = h_msgs[i];
         if (!dtype_ok(m.dtype) || (m.n > 0 && m.out == nullptr) ||
@@ -910,7 +923,7 @@ int zc_plan_decompress_streams(zc_batch* plan, int n_msgs, const void* const* h_
         it.raw_out = m.out;
         it.n = m.n;
         it.tile_begin = (unsigned)tile;
-        it.ntiles = (unsigned)tiles_for(m.n, DEC_U);
+        it.ntiles = (unsigned)tiles_for(m.n, du);
         it.chunk_begin = (unsigned)chunk;
         it.nchunks = it.ntiles <= local ? 0u : (unsigned)chunks_for(it.ntiles);
         it.x_dtype = m.dtype;
@@ -924,6 +937,7 @@ int zc_plan_decompress_streams(zc_batch* plan, int n_msgs, const void* const* h_
         return ZC_ERR_CUDA;
     std::memset(plan, 0, sizeof(*plan));
     plan->n_msgs = n_msgs;
+    plan->tile_chunks = du / 8;
     plan->decompress = 1;
     plan->total_tiles = tile;
     plan->total_chunks = chunk;
@@ -942,7 +956,7 @@ int zc_decompress_batch(const zc_batch* plan, void* d_ws, size_t ws_bytes, zc_st
     Launch P = base_launch(w);
     P.items = (const Item*)plan->d_table;
     P.n_items = (unsigned)plan->n_msgs;
-    P.urows = DEC_U;
+    P.urows = plan->tile_chunks == DEC_U_LARGE / 8 ? DEC_U_LARGE : DEC_U;
     P.in_base = (const uint8_t*)plan->d_packed;
     P.in_off = (const unsigned long long*)plan->d_msg_off;
     P.in_cap = plan->packed_cap;

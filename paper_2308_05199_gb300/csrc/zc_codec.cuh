@@ -27,7 +27,14 @@
 namespace zc {
 
 constexpr int WSCAN = NTHREADS;        // warp units per width-scan chunk
-constexpr int DEC_U = 64;              // rows per warp unit of the decompressor
+// Rows per warp unit of the decompressor.  A unit starts with a chain of three
+// round trips (header, width bytes and offset, payload), about a third of a
+// 64-row unit's time; large launches take 128-row units, small ones keep enough
+// CTAs with 64 (measured at 64 / 128: 2^27
+// elements of the field 126.5 / 124 us, 2^25 47.5 / 49.8, 2^26 BF16 gradients 75.3 / 73.2,
+// a batch of 250 messages 380 / 359).
+constexpr int DEC_U = 64;
+constexpr int DEC_U_LARGE = 128;
 // Batched decompression: items of at most this many decode tiles get no
 // width-scan chunks; their decoder CTAs find the unit offsets themselves.
 constexpr unsigned DEC_LOCAL_TILES = 4;
@@ -1324,11 +1331,12 @@ __global__ void __launch_bounds__(NTHREADS) k_wscan(const Launch P)
 // ---- decompression -------------------------------------------------------------
 
 // Raw streams: copy (and convert) the elements of this warp unit.
+template <int DU>
 __device__ __forceinline__ void unit_raw_copy(const Item& it, int src_dtype, unsigned long long ue0)
 {
     const uint8_t* src = it.cin + 32;
     const int lane = threadIdx.x & 31;
-    for (int r = 0; r < DEC_U; ++r) {
+    for (int r = 0; r < DU; ++r) {
         const unsigned long long e = ue0 + (unsigned long long)r * 32 + lane;
         if (e < it.n) {
             const float v = src_dtype == ZC_F32 ? __ldg((const float*)src + e)
@@ -1339,25 +1347,25 @@ __device__ __forceinline__ void unit_raw_copy(const Item& it, int src_dtype, uns
 }
 
 // One warp unit of a coded stream (zc_rows.cuh), 32 rows at a time.  `bufs`:
-// the warp's two group buffers; a group's payload arrives in its buffer (both
-// groups' copies are in flight before the first is decoded), and the decoded
-// rows take its place before they are stored, 16 bytes a lane.
+// the warp's two group buffers; a group's payload arrives in its buffer while the
+// group before it is decoded, and the decoded rows take its place before they are
+// stored, 16 bytes a lane.
 // off_local >= 0: the unit's payload offset found by the caller (a small
 // item's decoder CTA), in place of the width scan's P.offs[slot].
-template <int LOG2L, typename TO, bool HEADS = false>
+template <int LOG2L, typename TO, int DU, bool HEADS = false>
 __device__ __forceinline__ void unit_decode(const Launch& P, const Item& it, unsigned slot,
                                             unsigned long long ue0, float two_eb, unsigned bufs,
                                             long long off_local)
 {
-    static_assert(DEC_U == 2 * GROWS, "two groups per unit");
+    static_assert(DU % GROWS == 0, "whole groups");
     constexpr int L = 1 << LOG2L;
     constexpr int RPB = Blk<LOG2L>::RPB;
     const int lane = threadIdx.x & 31;
     const unsigned long long nb = (it.n + L - 1) >> LOG2L;
     const unsigned long long b0 = ue0 >> LOG2L;
-    const int un = (int)min(it.n - ue0, (unsigned long long)(DEC_U * 32));
-    const uint32_t wv1 = load_widths<LOG2L>(it.cin, nb, b0 + GELEMS / L);
-    const uint32_t wv0 = load_widths<LOG2L>(it.cin, nb, b0);
+    const int un = (int)min(it.n - ue0, (unsigned long long)(DU * 32));
+    uint32_t wn = load_widths<LOG2L>(it.cin, nb, b0 + GELEMS / L);
+    const uint32_t wv = load_widths<LOG2L>(it.cin, nb, b0);
     const bool slot_ok = off_local >= 0 || dcheck(P.ctl, slot < P.ws_cap, slot);
     unsigned long long pos = 32ull + ceil16(nb) + (HEADS ? ceil16(3ull * nb) : 0ull) +
                              (off_local >= 0 ? (unsigned long long)off_local
@@ -1388,11 +1396,23 @@ __device__ __forceinline__ void unit_decode(const Launch& P, const Item& it, uns
         pos += (unsigned long long)tot;
         return G;
     };
-    Group G = fetch(wv0, bufs), G1 = fetch(wv1, bufs + GBUF);
+    // Two groups: both copies before the first is decoded.  More: each group's
+    // copy while the one before it is decoded (two copies in flight throughout
+    // took more registers: 377 us for a batch that takes 359).
+    constexpr bool PAIR = DU == 2 * GROWS;
+    Group G = fetch(wv, bufs), G1 = G;
+    if (PAIR) G1 = fetch(wn, bufs + GBUF);
 #pragma unroll 1
     for (int g = 0; g * GELEMS < un; ++g) {
         const int nrem = min(un - g * GELEMS, GELEMS);
-        const unsigned buf = bufs + g * GBUF;
+        const unsigned buf = bufs + (g & 1) * GBUF;
+        if (!PAIR && (g + 1) * GELEMS < un) {
+            G1 = fetch(wn, bufs + ((g + 1) & 1) * GBUF);
+            if ((g + 2) * GELEMS < un)
+                wn = load_widths<LOG2L>(it.cin, nb, b0 + (unsigned)((g + 2) * (GELEMS / L)));
+        } else if (!PAIR) {
+            cp_commit();
+        }
         int h0 = 0, h16 = 0;
         if (HEADS) {  // the heads of this lane's blocks
             const unsigned long long b = b0 + (unsigned)(g * (GELEMS / L)) +
@@ -1401,7 +1421,7 @@ __device__ __forceinline__ void unit_decode(const Launch& P, const Item& it, uns
             if ((lane & (RPB - 1)) == 0 && b < nb) h0 = load_head(hp);
             if (L == 16 && b + 1 < nb) h16 = load_head(hp + 3);
         }
-        if (g == 0) cp_wait<1>();
+        if (!PAIR || g == 0) cp_wait<1>();
         else cp_wait<0>();
         __syncwarp();
         const PlaneSrc<true> ps{G.sp, nullptr};
@@ -1421,6 +1441,7 @@ __device__ __forceinline__ void unit_decode(const Launch& P, const Item& it, uns
         __syncwarp();
         TO* const op = (TO*)it.raw_out + ue0 + g * GELEMS;
         stage_out<TO>(op, nrem, ((uintptr_t)op & 15u) == 0, buf);
+        if (!PAIR) __syncwarp();  // the buffer is free
         G = G1;
     }
     cp_wait<0>();
@@ -1432,6 +1453,7 @@ __device__ __forceinline__ void unit_decode(const Launch& P, const Item& it, uns
 // offset; the item's last tile checks the total against the header's payload
 // size, as the width scan does.  Called by every thread of the CTA (coded
 // streams only: lg >= 4).
+template <int DU>
 __device__ __forceinline__ unsigned long long local_unit_offset(const Item& it, int lg, unsigned t,
                                                                 Ctl* ctl, unsigned item_idx)
 {
@@ -1440,7 +1462,7 @@ __device__ __forceinline__ unsigned long long local_unit_offset(const Item& it, 
     const int lgb = lg & 7;
     const unsigned long long PB = (1ull << lgb) / 8;
     const unsigned long long nb = (it.n + (1ull << lgb) - 1) >> lgb;
-    const unsigned bpu = (unsigned)(DEC_U * 32) >> lgb;  // blocks per unit: 16 to 128
+    const unsigned bpu = (unsigned)(DU * 32) >> lgb;  // blocks per unit: 16 to 256
     // width bytes, 16 at a time (the array is zero padded to 16; a unit and a
     // tile start at multiples of 16)
     const uint4* const w = (const uint4*)(it.cin + 32);
@@ -1475,7 +1497,7 @@ __device__ __forceinline__ unsigned long long local_unit_offset(const Item& it, 
 // BATCH: a multi-item launch; LOCAL: (some) items find their own unit offsets.
 // The decoder of a single scanned stream is compiled without that path, which
 // would cost it registers.
-template <bool BATCH, bool LOCAL>
+template <bool BATCH, bool LOCAL, int DU>
 __device__ __forceinline__ void decompress_tile(const Launch& P)
 {
     extern __shared__ __align__(128) uint8_t dsm[];
@@ -1503,14 +1525,14 @@ __device__ __forceinline__ void decompress_tile(const Launch& P)
     }
     const unsigned t = tile - it.tile_begin;
     const int warp = threadIdx.x >> 5;
-    const unsigned long long ue0 = ((unsigned long long)t * NWARPS + warp) * (DEC_U * 32);
+    const unsigned long long ue0 = ((unsigned long long)t * NWARPS + warp) * (DU * 32);
     const unsigned slot = tile * NWARPS + warp;
     const unsigned bufs = (unsigned)__cvta_generic_to_shared(dsm) + warp * (2 * GBUF);
     float eb_in;
     const int lg = check_header(it, P.ctl, idx, -1, eb_in, threadIdx.x == 0 && t == 0);
     long long loff = -1;  // the unit's payload offset, when this CTA finds it
     if (LOCAL && it.nchunks == 0 && lg >= 4)  // uniform in the CTA
-        loff = (long long)local_unit_offset(it, lg, t, P.ctl, idx);
+        loff = (long long)local_unit_offset<DU>(it, lg, t, P.ctl, idx);
     // the width scan's offsets are read from here on: a single-stream decoder
     // launched dependent on the scan has looked up its tile and checked the
     // header while the scan ran, and waits for it now.  Every thread passes
@@ -1521,37 +1543,37 @@ __device__ __forceinline__ void decompress_tile(const Launch& P)
     const float two = __fadd_rn(eb_in, eb_in);
     if (it.out_dtype == ZC_F32) {
         switch (lg) {
-        case 4: unit_decode<4, float>(P, it, slot, ue0, two, bufs, loff); return;
-        case 5: unit_decode<5, float>(P, it, slot, ue0, two, bufs, loff); return;
-        case 6: unit_decode<6, float>(P, it, slot, ue0, two, bufs, loff); return;
-        case 7: unit_decode<7, float>(P, it, slot, ue0, two, bufs, loff); return;
-        case 12: unit_decode<4, float, true>(P, it, slot, ue0, two, bufs, loff); return;
-        case 13: unit_decode<5, float, true>(P, it, slot, ue0, two, bufs, loff); return;
-        case 14: unit_decode<6, float, true>(P, it, slot, ue0, two, bufs, loff); return;
-        case 15: unit_decode<7, float, true>(P, it, slot, ue0, two, bufs, loff); return;
+        case 4: unit_decode<4, float, DU>(P, it, slot, ue0, two, bufs, loff); return;
+        case 5: unit_decode<5, float, DU>(P, it, slot, ue0, two, bufs, loff); return;
+        case 6: unit_decode<6, float, DU>(P, it, slot, ue0, two, bufs, loff); return;
+        case 7: unit_decode<7, float, DU>(P, it, slot, ue0, two, bufs, loff); return;
+        case 12: unit_decode<4, float, DU, true>(P, it, slot, ue0, two, bufs, loff); return;
+        case 13: unit_decode<5, float, DU, true>(P, it, slot, ue0, two, bufs, loff); return;
+        case 14: unit_decode<6, float, DU, true>(P, it, slot, ue0, two, bufs, loff); return;
+        case 15: unit_decode<7, float, DU, true>(P, it, slot, ue0, two, bufs, loff); return;
         default: break;
         }
     } else {
         switch (lg) {
-        case 4: unit_decode<4, uint16_t>(P, it, slot, ue0, two, bufs, loff); return;
-        case 5: unit_decode<5, uint16_t>(P, it, slot, ue0, two, bufs, loff); return;
-        case 6: unit_decode<6, uint16_t>(P, it, slot, ue0, two, bufs, loff); return;
-        case 7: unit_decode<7, uint16_t>(P, it, slot, ue0, two, bufs, loff); return;
-        case 12: unit_decode<4, uint16_t, true>(P, it, slot, ue0, two, bufs, loff); return;
-        case 13: unit_decode<5, uint16_t, true>(P, it, slot, ue0, two, bufs, loff); return;
-        case 14: unit_decode<6, uint16_t, true>(P, it, slot, ue0, two, bufs, loff); return;
-        case 15: unit_decode<7, uint16_t, true>(P, it, slot, ue0, two, bufs, loff); return;
+        case 4: unit_decode<4, uint16_t, DU>(P, it, slot, ue0, two, bufs, loff); return;
+        case 5: unit_decode<5, uint16_t, DU>(P, it, slot, ue0, two, bufs, loff); return;
+        case 6: unit_decode<6, uint16_t, DU>(P, it, slot, ue0, two, bufs, loff); return;
+        case 7: unit_decode<7, uint16_t, DU>(P, it, slot, ue0, two, bufs, loff); return;
+        case 12: unit_decode<4, uint16_t, DU, true>(P, it, slot, ue0, two, bufs, loff); return;
+        case 13: unit_decode<5, uint16_t, DU, true>(P, it, slot, ue0, two, bufs, loff); return;
+        case 14: unit_decode<6, uint16_t, DU, true>(P, it, slot, ue0, two, bufs, loff); return;
+        case 15: unit_decode<7, uint16_t, DU, true>(P, it, slot, ue0, two, bufs, loff); return;
         default: break;
         }
     }
-    if (lg == -2) unit_raw_copy(it, ZC_F32, ue0);
-    else if (lg == -3) unit_raw_copy(it, ZC_BF16, ue0);
+    if (lg == -2) unit_raw_copy<DU>(it, ZC_F32, ue0);
+    else if (lg == -3) unit_raw_copy<DU>(it, ZC_BF16, ue0);
 }
 
-template <bool BATCH, bool LOCAL>
+template <bool BATCH, bool LOCAL, int DU>
 __global__ void __launch_bounds__(NTHREADS, DEC_CTAS_PER_SM) k_decompress(const Launch P)
 {
-    decompress_tile<BATCH, LOCAL>(P);
+    decompress_tile<BATCH, LOCAL, DU>(P);
 }
 
 #endif  // ZC_DECODE_KERNELS

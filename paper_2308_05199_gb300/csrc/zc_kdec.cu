@@ -37,21 +37,22 @@ cudaError_t launch_group(Item* items, unsigned n_items, unsigned* part, unsigned
     return cudaGetLastError();
 }
 
-cudaError_t launch_decompress(const Launch& P, unsigned grid, cudaStream_t s, bool after_wscan)
+template <int DU>
+static cudaError_t decompress_u(const Launch& P, unsigned grid, cudaStream_t s, bool after_wscan)
 {
     if (P.items != nullptr) {
-        const cudaError_t e = smem_limit<k_decompress<true, true>>(DEC_SMEM_BYTES);
+        const cudaError_t e = smem_limit<k_decompress<true, true, DU>>(DEC_SMEM_BYTES);
         if (e != cudaSuccess) return e;
-        k_decompress<true, true><<<grid, NTHREADS, DEC_SMEM_BYTES, s>>>(P);
+        k_decompress<true, true, DU><<<grid, NTHREADS, DEC_SMEM_BYTES, s>>>(P);
         return cudaGetLastError();
     }
-    if (!after_wscan) {
-        const cudaError_t e = smem_limit<k_decompress<false, true>>(DEC_SMEM_BYTES);
+    if (!after_wscan) {  // (small streams only: 64-row units)
+        const cudaError_t e = smem_limit<k_decompress<false, true, DEC_U>>(DEC_SMEM_BYTES);
         if (e != cudaSuccess) return e;
-        k_decompress<false, true><<<grid, NTHREADS, DEC_SMEM_BYTES, s>>>(P);
+        k_decompress<false, true, DEC_U><<<grid, NTHREADS, DEC_SMEM_BYTES, s>>>(P);
         return cudaGetLastError();
     }
-    const cudaError_t e = smem_limit<k_decompress<false, false>>(DEC_SMEM_BYTES);
+    const cudaError_t e = smem_limit<k_decompress<false, false, DU>>(DEC_SMEM_BYTES);
     if (e != cudaSuccess) return e;
     // launched dependent on the width scan just before it on the stream: its
     // CTAs read their headers and width bytes while the scan still runs
@@ -65,7 +66,13 @@ cudaError_t launch_decompress(const Launch& P, unsigned grid, cudaStream_t s, bo
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_decompress<false, false>, P);
+    return cudaLaunchKernelEx(&cfg, k_decompress<false, false, DU>, P);
+}
+
+cudaError_t launch_decompress(const Launch& P, unsigned grid, cudaStream_t s, bool after_wscan)
+{
+    return P.urows == DEC_U_LARGE ? decompress_u<DEC_U_LARGE>(P, grid, s, after_wscan)
+                                  : decompress_u<DEC_U>(P, grid, s, after_wscan);
 }
 
 }  // namespace zc
