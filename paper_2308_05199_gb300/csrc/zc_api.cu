@@ -610,10 +610,12 @@ int zc_reduce_step_batch(const zc_plan* plan, void* d_ws, size_t ws_bytes, zc_st
     P.n_items = (unsigned)plan->n_items;
     P.urows = unit_rows(C);
     const bool scan = plan->has_input != 0 && plan->total_chunks > 0;
+    const bool chunk_map = scan && plan->n_items >= CHUNK_MAP_ITEMS;
     if (scan) {
         P.total_tiles = (unsigned)plan->total_chunks;
-        if (plan->n_items >= CHUNK_MAP_ITEMS) {
-            // chunk -> item map for the width scan (the tile map below reuses its space)
+        if (chunk_map) {
+            // chunk -> item map for the width scan (the tile map below reuses its
+            // space, so that one is then not built while the scan runs)
             if (launch_tile_map(P.items, P.n_items, P.total_tiles, w.tile_map, (cudaStream_t)s,
                                 true) != cudaSuccess)
                 return ZC_ERR_CUDA;
@@ -636,7 +638,7 @@ int zc_reduce_step_batch(const zc_plan* plan, void* d_ws, size_t ws_bytes, zc_st
     // 8192^2: 1685 us with maps, 1710 without).
     if (plan->n_items > (plan->total_tiles <= LOCAL_LAUNCH_TILES ? SEARCH_ITEMS : 1)) {
         if (launch_tile_map(P.items, P.n_items, P.total_tiles, w.tile_map, (cudaStream_t)s,
-                            false, scan) != cudaSuccess)
+                            false, scan && !chunk_map) != cudaSuccess)
             return ZC_ERR_CUDA;
         P.tile_map = w.tile_map;
         P.dep = 1;
