@@ -641,9 +641,6 @@ int zc_reduce_step_batch(const zc_plan* plan, void* d_ws, size_t ws_bytes, zc_st
                             false, scan && !chunk_map) != cudaSuccess)
             return ZC_ERR_CUDA;
         P.tile_map = w.tile_map;
-        P.dep = 1;
-    } else {
-        P.dep = scan;
     }
     return cuda_status(launch_reduce_any(lg, C, P, (unsigned)grid, (cudaStream_t)s));
 }

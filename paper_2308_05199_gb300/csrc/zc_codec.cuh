@@ -105,10 +105,6 @@ struct Launch {
     // order, so seg_off[i] is only item i's start and seg_off[n_items] the
     // packed total; a decoder bounds a stream by seg_off[n_items]
     int grouped;
-    // encoder launches: launched dependent on the kernel just before on the
-    // stream (programmatic serialisation), whose results the CTAs wait for
-    // in their prologue (a relative bound, eb_from_ctl, implies it)
-    int dep;
 };
 
 struct Smem {
@@ -878,17 +874,20 @@ __device__ __forceinline__ void enc_pipeline(const Launch& P, const Src& src, En
     __shared__ EncShared es;
     extern __shared__ __align__(128) uint8_t dsm[];  // group buffers, width bytes [slot][warp][2U]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // a relative bound comes from the range kernel launched just before, the
-    // fused ring step's offsets and tile map from the kernels before it: an
-    // encoder launched dependent on them waits here for them to complete
-    // (every thread: their results are read below and in every tile)
-    if (P.eb_from_ctl || P.dep) grid_dep_wait();
+    // every thread: what the kernels before wrote (a relative bound, offsets,
+    // the tile map) is read below and in every tile
+    grid_dep_wait();
+    grid_dep_launch();
+    const unsigned modulus = P.total_tiles + gridDim.x - 1u;
+    const bool rings = (unsigned long long)gridDim.x * ring_cta_bytes(U) <= P.ring_bytes;
+    unsigned g0 = 0u;  // thread 0: the first ticket, taken with the control block's words
     if (tid == 0) {
+        if (rings) g0 = atomicInc(&P.ctl->ticket, modulus);
         es.E = ld_volatile_u32(&P.ctl->epoch) + 1u;
         int a = ld_volatile_u32(&P.ctl->magic) != WS_MAGIC;
         if (a) {
             fail(P.ctl, ZC_ERR_WORKSPACE, 0);
-        } else if ((unsigned long long)gridDim.x * ring_cta_bytes(U) > P.ring_bytes) {
+        } else if (!rings) {
             a = 1;  // more CTAs than rings: the whole launch does nothing
             if (blockIdx.x == 0) fail(P.ctl, ZC_ERR_WORKSPACE, 1);
         } else if (P.eb_from_ctl && ld_volatile_u32(&P.ctl->eb_ok) != 1u) {
@@ -900,7 +899,6 @@ __device__ __forceinline__ void enc_pipeline(const Launch& P, const Src& src, En
     if (es.abort == 1) return;
     const bool no_eb = es.abort == 2;
     const unsigned E = es.E;
-    const unsigned modulus = P.total_tiles + gridDim.x - 1u;
     uint8_t* const ring = P.ring + (unsigned long long)blockIdx.x * ring_cta_bytes(U);
     if (warp < NWARPS) {
         auto seg_of = [&](int s) { return ring + (unsigned long long)(s * NWARPS + warp) * seg_bytes(U); };
@@ -919,7 +917,7 @@ __device__ __forceinline__ void enc_pipeline(const Launch& P, const Src& src, En
             bar_sync_n(BAR_ENCW, NTHREADS);  // slot s's previous tile is stored
             if (tid == 0) {
                 TileSlot& S = slots[s];
-                const unsigned g = atomicInc(&P.ctl->ticket, modulus);
+                const unsigned g = i == 0 ? g0 : atomicInc(&P.ctl->ticket, modulus);
                 S.g = g;
                 S.valid = g < P.total_tiles;
                 S.item = g < P.total_tiles ? src.find(g) : 0u;
@@ -1226,6 +1224,7 @@ __global__ void __launch_bounds__(NTHREADS) k_wscan(const Launch P)
 {
     __shared__ Smem sm;
     __shared__ int wsum[NWARPS];
+    grid_dep_wait();
     grid_dep_launch();  // the decoder after it may be launched now (it waits for the offsets)
     const unsigned modulus = P.total_tiles + gridDim.x - 1u;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1501,6 +1500,8 @@ template <bool BATCH, bool LOCAL, int DU>
 __device__ __forceinline__ void decompress_tile(const Launch& P)
 {
     extern __shared__ __align__(128) uint8_t dsm[];
+    if (BATCH || LOCAL) grid_dep_wait();
+    grid_dep_launch();
     const unsigned tile = blockIdx.x;
     unsigned idx = 0;
     if (P.tile_map != nullptr) {

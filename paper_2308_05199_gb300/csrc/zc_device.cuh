@@ -119,6 +119,13 @@ __device__ __forceinline__ unsigned long long ceil16(unsigned long long v)
 // runs; grid_dep_wait() blocks until that kernel has completed and its memory
 // operations are visible (it returns at once in a kernel launched without
 // the attribute).  grid_dep_launch() lets the dependent kernel start early.
+// The codec's kernels (but the range pass) are launched this way and call both
+// first thing, in this order: the launch of a kernel, and its CTAs' way onto the
+// SMs, overlap the end of the one before (a 4 MiB signal, there and back: 23.1 ->
+// 19.9 us; five-rank recursive doubling of 1M elements: 118 -> 113).  A kernel that lets the next one
+// start only after its own wait keeps every kernel before it complete, so
+// what the next one reads ahead of its own wait (the decoder its stream's
+// header, the tile map its items) is not still being written.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

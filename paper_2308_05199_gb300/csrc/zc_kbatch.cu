@@ -15,8 +15,7 @@ cudaError_t launch_batch_u(const Launch& P, unsigned grid, cudaStream_t s)
 {
     const cudaError_t e = smem_limit<k_batch<U>>(enc_smem_bytes(U));
     if (e != cudaSuccess) return e;
-    k_batch<U><<<grid, ENC_THREADS, enc_smem_bytes(U), s>>>(P);
-    return cudaGetLastError();
+    return launch_after(k_batch<U>, grid, ENC_THREADS, enc_smem_bytes(U), s, P);
 }
 
 template cudaError_t launch_batch_u<ZC_BATCH_U>(const Launch&, unsigned, cudaStream_t);

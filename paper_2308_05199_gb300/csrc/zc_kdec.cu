@@ -6,25 +6,16 @@ namespace zc {
 
 cudaError_t launch_wscan(const Launch& P, unsigned grid, cudaStream_t s)
 {
-    k_wscan<<<grid, NTHREADS, 0, s>>>(P);
-    return cudaGetLastError();
+    return launch_after(k_wscan, grid, NTHREADS, 0, s, P);
 }
 
 cudaError_t launch_tile_map(const Item* items, unsigned n_items, unsigned total_tiles,
                             unsigned* map, cudaStream_t s, bool by_chunk, bool dependent)
 {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((total_tiles + NTHREADS - 1) / NTHREADS);
-    cfg.blockDim = dim3(NTHREADS);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = dependent ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k_tile_map, items, n_items, total_tiles, map,
-                              by_chunk ? 1 : 0);
+    const unsigned grid = (total_tiles + NTHREADS - 1) / NTHREADS;
+    if (dependent) return launch_after(k_tile_map, grid, NTHREADS, 0, s, items, n_items, total_tiles, map, by_chunk ? 1 : 0);
+    k_tile_map<<<grid, NTHREADS, 0, s>>>(items, n_items, total_tiles, map, by_chunk ? 1 : 0);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_group(Item* items, unsigned n_items, unsigned* part, unsigned* map,
@@ -43,30 +34,18 @@ static cudaError_t decompress_u(const Launch& P, unsigned grid, cudaStream_t s, 
     if (P.items != nullptr) {
         const cudaError_t e = smem_limit<k_decompress<true, true, DU>>(DEC_SMEM_BYTES);
         if (e != cudaSuccess) return e;
-        k_decompress<true, true, DU><<<grid, NTHREADS, DEC_SMEM_BYTES, s>>>(P);
-        return cudaGetLastError();
+        return launch_after(k_decompress<true, true, DU>, grid, NTHREADS, DEC_SMEM_BYTES, s, P);
     }
     if (!after_wscan) {  // (small streams only: 64-row units)
         const cudaError_t e = smem_limit<k_decompress<false, true, DEC_U>>(DEC_SMEM_BYTES);
         if (e != cudaSuccess) return e;
-        k_decompress<false, true, DEC_U><<<grid, NTHREADS, DEC_SMEM_BYTES, s>>>(P);
-        return cudaGetLastError();
+        return launch_after(k_decompress<false, true, DEC_U>, grid, NTHREADS, DEC_SMEM_BYTES, s, P);
     }
     const cudaError_t e = smem_limit<k_decompress<false, false, DU>>(DEC_SMEM_BYTES);
     if (e != cudaSuccess) return e;
     // launched dependent on the width scan just before it on the stream: its
     // CTAs read their headers and width bytes while the scan still runs
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(NTHREADS);
-    cfg.dynamicSmemBytes = DEC_SMEM_BYTES;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_decompress<false, false, DU>, P);
+    return launch_after(k_decompress<false, false, DU>, grid, NTHREADS, DEC_SMEM_BYTES, s, P);
 }
 
 cudaError_t launch_decompress(const Launch& P, unsigned grid, cudaStream_t s, bool after_wscan)

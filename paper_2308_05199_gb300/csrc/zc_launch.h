@@ -24,6 +24,26 @@ inline cudaError_t smem_limit(int bytes)
     return e;
 }
 
+// Launches a kernel that begins with grid_dep_wait() dependent on the kernel
+// just before it on the stream (programmatic serialisation; nothing changes
+// where the work before it is not a kernel).
+template <typename... A>
+inline cudaError_t launch_after(void (*k)(A...), unsigned grid, unsigned threads, int smem, cudaStream_t s,
+                                const A&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 // Launchers of the encoder kernels at block size 2^LG; each is defined and
 // explicitly instantiated by the object of zc_kenc.cu built for that LG.
 // `chunks` is the tile size in 2048-element chunks (4, 8 or 16); these pick

@@ -208,6 +208,9 @@ __global__ void k_ws_init(Ctl* c)
 
 cudaError_t launch_range(const RangeLaunch& R, unsigned grid, cudaStream_t s)
 {
+    // Not dependent on the kernel before: its CTAs share the input out evenly,
+    // and placed on the SMs as those come free from that kernel's last CTAs, some
+    // SMs got many of them (512^3 field, range and compression: 221 -> 240 us).
     if (R.dtype == ZC_F32) k_range_one<float><<<grid, 256, 0, s>>>(R);
     else k_range_one<uint16_t><<<grid, 256, 0, s>>>(R);
     return cudaGetLastError();
