@@ -1109,6 +1109,8 @@ __device__ __forceinline__ int group_class(int log2L) { return log2L < 4 ? 0 : l
 __global__ void __launch_bounds__(GROUP_T) k_group_count(const Item* items, unsigned n_items,
                                                          unsigned* part)
 {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ unsigned red[GROUP_CLASSES][GROUP_T / 32];
     const unsigned i = blockIdx.x * GROUP_T + threadIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1136,6 +1138,8 @@ __global__ void __launch_bounds__(GROUP_T) k_group_count(const Item* items, unsi
 // of all smaller classes) plus the class's tiles in CTAs before b.
 __global__ void __launch_bounds__(1024) k_group_scan(unsigned* part, unsigned nblk)
 {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ unsigned wsum[32];
     __shared__ unsigned carry[GROUP_CLASSES];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1183,6 +1187,8 @@ __global__ void __launch_bounds__(1024) k_group_scan(unsigned* part, unsigned nb
 __global__ void __launch_bounds__(GROUP_T) k_group_place(Item* items, unsigned n_items,
                                                          const unsigned* part, unsigned* map)
 {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ unsigned wsum[GROUP_CLASSES][GROUP_T / 32];
     const unsigned i = blockIdx.x * GROUP_T + threadIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

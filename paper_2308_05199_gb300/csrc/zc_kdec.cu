@@ -22,10 +22,11 @@ cudaError_t launch_group(Item* items, unsigned n_items, unsigned* part, unsigned
                          cudaStream_t s)
 {
     const unsigned nblk = (n_items + GROUP_T - 1) / GROUP_T;
-    k_group_count<<<nblk, GROUP_T, 0, s>>>(items, n_items, part);
-    k_group_scan<<<1, 1024, 0, s>>>(part, nblk);
-    k_group_place<<<nblk, GROUP_T, 0, s>>>(items, n_items, part, map);
-    return cudaGetLastError();
+    const cudaError_t e1 = launch_after(k_group_count, nblk, GROUP_T, 0, s, (const Item*)items, n_items, part);
+    if (e1 != cudaSuccess) return e1;
+    const cudaError_t e2 = launch_after(k_group_scan, 1, 1024, 0, s, part, nblk);
+    if (e2 != cudaSuccess) return e2;
+    return launch_after(k_group_place, nblk, GROUP_T, 0, s, items, n_items, (const unsigned*)part, map);
 }
 
 template <int DU>

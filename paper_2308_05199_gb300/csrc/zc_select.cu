@@ -174,6 +174,8 @@ __device__ __forceinline__ unsigned stat_span(const float v[4], int cnt, const I
 __global__ void __launch_bounds__(256, 4) k_chunk_stats(const Item* items, unsigned n_items,
                                                      float* feat)
 {
+    grid_dep_wait();
+    grid_dep_launch();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned idx = blockIdx.x * 8 + warp;
     if (idx >= n_items) return;  // warp-uniform; only warp-level sync below
@@ -420,6 +422,8 @@ __device__ __forceinline__ void mlp_forward_tile(MlpSmem& sm)
 __global__ void __launch_bounds__(MT) k_mlp_forward(const float* P, const float* norm,
                                                     const float* X, int B, float* Yout)
 {
+    grid_dep_wait();
+    grid_dep_launch();
     extern __shared__ __align__(16) uint8_t raw[];
     MlpSmem& sm = *reinterpret_cast<MlpSmem*>(raw);
     const int ntiles = (B + TB - 1) / TB;
@@ -955,6 +959,8 @@ struct SelectArgs {
 __global__ void k_select(Item* items, unsigned n_items, const float* feat, const float* pred,
                          const float* pred_time, SelectArgs a, int* choice, unsigned* counts)
 {
+    grid_dep_wait();
+    grid_dep_launch();
     const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_items) return;
     Item& it = items[i];
@@ -1020,8 +1026,10 @@ int zc_batch_chunk_stats(const zc_batch* plan, float* d_feat, zc_stream_t s)
         d_feat == nullptr || (reinterpret_cast<uintptr_t>(d_feat) & 3) != 0)
         return ZC_ERR_ARG;
     const unsigned n = (unsigned)plan->n_msgs;
-    k_chunk_stats<<<(n + 7) / 8, 256, 0, (cudaStream_t)s>>>((const Item*)plan->d_table, n, d_feat);
-    return cudaGetLastError() == cudaSuccess ? ZC_OK : ZC_ERR_CUDA;
+    return launch_after(k_chunk_stats, (n + 7) / 8, 256, 0, (cudaStream_t)s, (const Item*)plan->d_table, n,
+                        d_feat) == cudaSuccess
+               ? ZC_OK
+               : ZC_ERR_CUDA;
 }
 
 static cudaError_t mlp_prepare()
@@ -1045,8 +1053,10 @@ int zc_mlp_forward(const float* d_params, const float* d_norm, const float* d_x,
         return ZC_ERR_CUDA;
     const int ntiles = (B + TB - 1) / TB;
     const int grid = ntiles < 2 * n_sm ? ntiles : 2 * n_sm;
-    k_mlp_forward<<<grid, MT, sizeof(MlpSmem), (cudaStream_t)s>>>(d_params, d_norm, d_x, B, d_y);
-    return cudaGetLastError() == cudaSuccess ? ZC_OK : ZC_ERR_CUDA;
+    return launch_after(k_mlp_forward, (unsigned)grid, MT, (int)sizeof(MlpSmem), (cudaStream_t)s, d_params,
+                        d_norm, d_x, B, d_y) == cudaSuccess
+               ? ZC_OK
+               : ZC_ERR_CUDA;
 }
 
 size_t zc_mlp_scratch_bytes(int B)
@@ -1146,9 +1156,10 @@ int zc_batch_select_timed(const zc_batch* plan, const float* d_feat, const float
         cudaMemsetAsync(d_counts, 0, 2 * sizeof(unsigned), (cudaStream_t)s) != cudaSuccess)
         return ZC_ERR_CUDA;
     const unsigned n = (unsigned)plan->n_msgs;
-    k_select<<<(n + 255) / 256, 256, 0, (cudaStream_t)s>>>((Item*)plan->d_table, n, d_feat, d_pred,
-                                                           d_pred_time, a, d_choice, d_counts);
-    return cudaGetLastError() == cudaSuccess ? ZC_OK : ZC_ERR_CUDA;
+    return launch_after(k_select, (n + 255) / 256, 256, 0, (cudaStream_t)s, (Item*)plan->d_table, n, d_feat,
+                        d_pred, d_pred_time, a, d_choice, d_counts) == cudaSuccess
+               ? ZC_OK
+               : ZC_ERR_CUDA;
 }
 
 int zc_batch_select(const zc_batch* plan, const float* d_feat, const float* d_pred,
