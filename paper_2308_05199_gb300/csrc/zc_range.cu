@@ -181,6 +181,7 @@ __device__ void range_finish(const RangeLaunch& P, Acc a)
 template <typename TX>
 __global__ void __launch_bounds__(256) k_range_one(const RangeLaunch P)
 {
+    grid_dep_wait();
     grid_dep_launch();  // the compressor after it may be launched now (it waits for the bound)
     Acc a{FLT_MAX, -FLT_MAX, false};
     const unsigned long long gtid = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -192,6 +193,7 @@ __global__ void __launch_bounds__(256) k_range_one(const RangeLaunch P)
 template <typename TX>
 __global__ void __launch_bounds__(256) k_range_multi(const RangeLaunch P, const RangeSegs S)
 {
+    grid_dep_wait();
     grid_dep_launch();  // the scatter pack after it may be launched now (it waits for the bound)
     Acc a{FLT_MAX, -FLT_MAX, false};
     const unsigned long long gtid = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -206,11 +208,17 @@ __global__ void k_ws_init(Ctl* c)
     c->magic = WS_MAGIC;
 }
 
+constexpr unsigned RANGE_SMALL_GRID = 152;  // at most a CTA per SM (1.2M elements)
+
 cudaError_t launch_range(const RangeLaunch& R, unsigned grid, cudaStream_t s)
 {
-    // Not dependent on the kernel before: its CTAs share the input out evenly,
-    // and placed on the SMs as those come free from that kernel's last CTAs, some
-    // SMs got many of them (512^3 field, range and compression: 221 -> 240 us).
+    // Dependent on the kernel before only while it is small: its CTAs share the
+    // input out evenly, and placed on the SMs as those come free from that
+    // kernel's last CTAs, some SMs get many of them (512^3 field, range and
+    // compression: 221 -> 240 us).
+    if (grid <= RANGE_SMALL_GRID)
+        return R.dtype == ZC_F32 ? launch_after(k_range_one<float>, grid, 256, 0, s, R)
+                                 : launch_after(k_range_one<uint16_t>, grid, 256, 0, s, R);
     if (R.dtype == ZC_F32) k_range_one<float><<<grid, 256, 0, s>>>(R);
     else k_range_one<uint16_t><<<grid, 256, 0, s>>>(R);
     return cudaGetLastError();

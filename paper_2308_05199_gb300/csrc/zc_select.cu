@@ -1092,6 +1092,24 @@ int zc_mlp_sgd(float* d_params, float* d_vel, const float* d_grad, float lr, flo
     return cudaGetLastError() == cudaSuccess ? ZC_OK : ZC_ERR_CUDA;
 }
 
+// Whether the current device runs a cluster of this launch (a partition of a GPU
+// may have no room for one of this size); asked once per device.
+static bool fit_cluster(const cudaLaunchConfig_t& cfg)
+{
+    static std::atomic<int> known[64];  // 0: not asked, 1: yes, 2: no
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::atomic<int>* const k = dev >= 0 && dev < 64 ? &known[dev] : nullptr;
+    if (k != nullptr && k->load(std::memory_order_acquire) != 0) return k->load(std::memory_order_acquire) == 1;
+    int clusters = 0;
+    const bool ok = smem_limit<k_mlp_fit>((int)sizeof(FitSmem)) == cudaSuccess &&
+                    cudaFuncSetAttribute(k_mlp_fit, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&clusters, k_mlp_fit, &cfg) == cudaSuccess && clusters > 0;
+    if (!ok) cudaGetLastError();
+    if (k != nullptr) k->store(ok ? 1 : 2, std::memory_order_release);
+    return ok;
+}
+
 int zc_mlp_fit_epoch(float* d_params, float* d_vel, float* d_grad, const float* d_norm,
                      const float* d_x, const float* d_t, const int* d_idx, int N, int batch,
                      double lr, double momentum, float* d_losses, void* d_scratch,
@@ -1115,13 +1133,7 @@ int zc_mlp_fit_epoch(float* d_params, float* d_vel, float* d_grad, const float* 
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    // (a partition of the GPU may have no room for a cluster of this size)
-    int clusters = 0;
-    bool fits = batch <= FIT_MAX_BATCH && smem_limit<k_mlp_fit>((int)sizeof(FitSmem)) == cudaSuccess &&
-                cudaFuncSetAttribute(k_mlp_fit, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                cudaOccupancyMaxActiveClusters(&clusters, k_mlp_fit, &cfg) == cudaSuccess && clusters > 0;
-    if (!fits) {
-        cudaGetLastError();
+    if (batch > FIT_MAX_BATCH || !fit_cluster(cfg)) {
         for (int m = 0; (long long)m * batch < N; ++m) {
             const int B = N - m * batch < batch ? N - m * batch : batch;
             int st = zc_mlp_grad(d_params, d_norm, d_x, d_t, d_idx + (size_t)m * batch, B, d_grad,

@@ -492,8 +492,9 @@ def scatter_pack(x: torch.Tensor, counts, displs, eb: float, block: int = 32, mo
     x = x.contiguous()
     P = len(counts)
     ws = ws or Workspace(int(sum(counts)), P, x.device, stream)
-    cap = sum(zc_max_compressed_bytes(int(c), block) for c in counts)
-    out = out if out is not None else torch.empty(cap, dtype=torch.uint8, device=x.device)
+    if out is None:
+        cap = sum(zc_max_compressed_bytes(int(c), block) for c in counts)
+        out = torch.empty(cap, dtype=torch.uint8, device=x.device)
     seg_off = seg_off if seg_off is not None else torch.zeros(P + 1, dtype=torch.int64,
                                                               device=x.device)
     hc = (ctypes.c_uint64 * P)(*[int(c) for c in counts])
