@@ -20,8 +20,6 @@
 // units); decoding then needs no look-back and no barrier.
 #pragma once
 
-#include <type_traits>
-
 #include "zc_rows.cuh"
 
 namespace zc {
@@ -109,10 +107,8 @@ struct Launch {
 
 struct Smem {
     LbSmem lb;
-    unsigned long long base, start, end;
     unsigned ticket, item, E;
-    int abort, hdr_lg;
-    float eb, two_eb, inv;
+    int abort;
 };
 
 // Encoder CTAs: NWARPS encoder warps plus one resolver warp, enc_slots(U)
@@ -156,13 +152,6 @@ __device__ __forceinline__ int warp_excl_scan(int v, int lane, int& total)
     }
     total = __shfl_sync(FULL, s, 31);
     return s - v;
-}
-
-__device__ __forceinline__ int warp_sum(int v)
-{
-#pragma unroll
-    for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
-    return v;
 }
 
 // Reads and checks an input stream header for `it`; returns its log2 L (plus

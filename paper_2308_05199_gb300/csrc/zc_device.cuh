@@ -2,8 +2,7 @@
 //
 // Control block, status word, memory-ordering helpers, the bounded
 // decoupled look-back that turns per-tile byte counts into stream offsets in
-// one pass, the warp bit-matrix transpose that builds bit planes, and the
-// exact prequantizer.  Everything here is sm_103a CUDA; nothing is shared with
+// one pass, and the exact prequantizer.  Everything here is sm_103a CUDA; nothing is shared with
 // the CPU oracle.
 #pragma once
 
@@ -17,7 +16,6 @@ namespace zc {
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int NWARPS = 8;                  // warps per CTA
 constexpr int NTHREADS = NWARPS * 32;      // threads per CTA
-constexpr int MIN_ROWS = 4;                // smallest rows-per-warp: tile = 1024 elements
 constexpr unsigned WS_MAGIC = 0x5a435753u; // "ZCWS"
 constexpr int RANGE_SLOTS = 4096;          // partial min/max slots of the range kernel
 constexpr uint64_t WS_CTL_BYTES = 256;
@@ -41,34 +39,6 @@ static_assert(sizeof(Ctl) <= WS_CTL_BYTES, "control block too large");
 
 // ---- memory-ordering helpers -------------------------------------------
 
-__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p)
-{
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_release(unsigned long long* p, unsigned long long v)
-{
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p)
-{
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v)
-{
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-// Acquire fence: a relaxed load that observed a value written by a release
-// store, followed by this fence, sees everything written before that store.
-// Polling with relaxed loads and fencing once after the last one keeps the
-// (costly) acquire out of the polling loops.
-__device__ __forceinline__ void fence_acquire_gpu()
-{
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");
-}
 __device__ __forceinline__ unsigned ld_volatile_u32(const unsigned* p)
 {
     return *(const volatile unsigned*)p;
@@ -171,19 +141,7 @@ __device__ __forceinline__ bool quantize_fast(float x, float inv, int& q)
     return __fmaf_rn(fabsf(v), 2.384185791015625e-07f, f) < 0.5f;  // |v| * 2^-22
 }
 
-// The same, returning the bit pattern of the rounded float (q + QBIAS):
-// differences of two such values are differences of q, so an encoder that
-// only needs deltas skips the offset.
 constexpr int QBIAS = 0x4b400000;  // the bits of 1.5 * 2^23, the rounding constant
-__device__ __forceinline__ bool quantize_fast_bits(float x, float inv, int& qb)
-{
-    const float v = __fmul_rn(x, inv);
-    const float t = __fadd_rn(v, 12582912.0f);
-    const float r = __fsub_rn(t, 12582912.0f);
-    const float f = fabsf(__fsub_rn(v, r));
-    qb = __float_as_int(t);
-    return __fmaf_rn(fabsf(v), 2.384185791015625e-07f, f) < 0.5f;  // |v| * 2^-22
-}
 
 __device__ __forceinline__ int quantize(float x, float eb, float two_eb, float inv, int& q)
 {
