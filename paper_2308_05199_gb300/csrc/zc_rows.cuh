@@ -501,7 +501,9 @@ __device__ __noinline__ int encode_rows_general(const EncArgs A, unsigned bad, b
         if (L == 16 && i >= 16) o2 |= a;
         else o1 |= a;
     }
-    int np = o1 ? 33 - __clz(o1) : 0, np2 = L == 16 && o2 ? 33 - __clz(o2) : 0;
+    // (levels lie within 2^22, so deltas fit; a row's place is for no more planes)
+    int np = o1 ? min(33 - __clz(o1), ZC_MAX_WIDTH + 1) : 0;
+    int np2 = L == 16 && o2 ? min(33 - __clz(o2), ZC_MAX_WIDTH + 1) : 0;
     if ((lane & ~(RPB - 1)) * 32 >= A.nrem) np = 0;
     if (L == 16 && lane * 32 + 16 >= A.nrem) np2 = 0;
     const int npmax = __reduce_max_sync(FULL, max(np, np2));
@@ -582,6 +584,7 @@ __device__ __forceinline__ int encode_rows(const EncArgs& A, int& err)
     }
     uint32_t C[16];  // U_j, then the biased deltas of elements j and j + 16
     float me = 0.0f, mr = 0.0f;
+    bool jump = false;  // heads apart: more than 16 bits between this row and the one before
     int t0 = 0, t16 = 0, t31 = 0;
     uint32_t u0 = 0, up = 0;
     if (sizeof(T) == 4) {
@@ -651,8 +654,9 @@ __device__ __forceinline__ int encode_rows(const EncArgs& A, int& err)
             const int prev = __shfl_up_sync(FULL, t31, 1);
             if ((lane & (RPB - 1)) != 0) {
                 fill = prev;
-                // heads apart: only differences within a row are bounded so far
-                if (HEADS && abs(t0 - prev) >= 16000) mr = QLIM;
+                // heads apart: only differences within a row are bounded so far.
+                // (A flag of its own: mr tells apart what the row itself holds.)
+                if (HEADS) jump = (uint32_t)t0 - (uint32_t)prev + 15999u > 31998u;
             }
         }
         uint32_t um;
@@ -662,7 +666,7 @@ __device__ __forceinline__ int encode_rows(const EncArgs& A, int& err)
     }
     const bool far = !(mr < 1048576.0f) || (HEADS && !(fabsf(ref) < 1048576.0f));
     const bool bad = !(me < A.eb) || far;
-    if (__any_sync(FULL, bad || !(mr < QLIM)))
+    if (__any_sync(FULL, bad || jump || !(mr < QLIM)))
         return encode_rows_general<LOG2L, HEADS, sizeof(T) == 2>(A, __ballot_sync(FULL, bad),
                                                                  __any_sync(FULL, far), &err);
     if (HEADS) put_heads<LOG2L>(A, t0, t16);
