@@ -445,9 +445,9 @@ __device__ __forceinline__ void expand_bf16(unsigned buf)
 // The general path of a group: any width, any rounding, errors.  `bad`: rows
 // that hold a value whose fast rounding is not proven (near a tie, or beyond
 // 2^20: `far`).  Bad rows are requantized exactly, a lane per element, and
-// their values replaced by q 2eb, whose fast rounding is q again (|q| < 2^20:
-// x' and inv are off by at most 2^-24 relatively, so x' inv is within 1/8 of
-// q); with `far` set every row is requantized and the buffer then holds the
+// their values replaced by q 2eb, whose fast rounding is q again (|q| < 2^20,
+// heads apart 2^21: x' and inv are off by at most 2^-24 relatively, so x' inv is
+// within 1/4 of q); with `far` set every row is requantized and the buffer then holds the
 // rounding results themselves.  Then 32-bit deltas, byte by byte.  Not
 // inlined: a few groups in a hundred come here (near-tie values, |q| >=
 // 16000), and the fast path keeps its registers.
@@ -457,6 +457,9 @@ __device__ __noinline__ int encode_rows_general(const EncArgs A, unsigned bad, b
     constexpr int L = Blk<LOG2L>::L, RPB = Blk<LOG2L>::RPB;
     const int lane = threadIdx.x & 31;
     if (BF) expand_bf16(A.buf);
+    // q 2eb of a value near FLT_MAX may overflow (x = FLT_MAX, 2eb = 1.5 2^126: q =
+    // 3); |q| < 2^21 keeps it finite for a 2eb below 2^107
+    if (A.two_eb >= 0x1p107f) far = true;
     unsigned todo = far ? FULL : bad;
     while (todo) {  // warp-uniform
         const int r = __ffs(todo) - 1;
