@@ -158,20 +158,24 @@ __device__ __forceinline__ int warp_excl_scan(int v, int lane, int& total)
 // 8 when its block heads are stored apart), -1 for a format error (reported
 // when `report`), -2 / -3 for a raw FP32 / BF16 stream.  A caller that names
 // the block size it expects (the fused ring step) takes plain streams only.
+// WHOLE: the stream was complete before the kernel started (the scanned decoder:
+// the width scan before it has waited for it), so the loads may be non-coherent.
+template <bool WHOLE = false>
 __device__ __forceinline__ int check_header(const Item& it, Ctl* ctl, unsigned item_idx,
                                             int expect_log2L, float& eb_in, bool report)
 {
     const uint8_t* s = it.cin;
+    auto ld = [](const auto* p) { return WHOLE ? __ldg(p) : ld_dep(p); };
     if (it.cin_cap < 32) {
         if (report) fail(ctl, ZC_ERR_FORMAT, item_idx);
         return -1;
     }
-    const uint32_t w0 = __ldg((const unsigned*)s);
-    const uint32_t w1 = __ldg((const unsigned*)s + 1);
-    const unsigned long long n = __ldg((const unsigned long long*)s + 1);
-    eb_in = __uint_as_float(__ldg((const unsigned*)s + 4));
-    const uint32_t nb = __ldg((const unsigned*)s + 5);
-    const unsigned long long payload = __ldg((const unsigned long long*)s + 3);
+    const uint32_t w0 = ld((const unsigned*)s);
+    const uint32_t w1 = ld((const unsigned*)s + 1);
+    const unsigned long long n = ld((const unsigned long long*)s + 1);
+    eb_in = __uint_as_float(ld((const unsigned*)s + 4));
+    const uint32_t nb = ld((const unsigned*)s + 5);
+    const unsigned long long payload = ld((const unsigned long long*)s + 3);
     const int dtype = w1 & 0xff, lg = (w1 >> 8) & 0xff, flags = (w1 >> 16) & 0xff;
     bool ok = w0 == 0x3176435au && (w1 >> 24) == 0u && (dtype == 0 || dtype == 1) &&
               (flags & ~3) == 0 && flags != 3 && n == it.n;
@@ -204,8 +208,8 @@ __device__ __forceinline__ int planes_of(int w) { return w ? w + 1 : 0; }
 // Block head of the heads-apart format: 24-bit two's complement, little-endian.
 __device__ __forceinline__ int load_head(const uint8_t* p)
 {
-    const unsigned v = (unsigned)__ldg(p) | ((unsigned)__ldg(p + 1) << 8) |
-                       ((unsigned)__ldg(p + 2) << 16);
+    const unsigned v = (unsigned)ld_dep(p) | ((unsigned)ld_dep(p + 1) << 8) |
+                       ((unsigned)ld_dep(p + 2) << 16);
     return (int)v - ((v & 0x800000u) ? (1 << 24) : 0);
 }
 
@@ -220,8 +224,8 @@ __device__ __forceinline__ uint32_t load_widths(const uint8_t* cin, unsigned lon
     const unsigned long long b =
         bg + (LOG2L == 4 ? 2u * lane : LOG2L == 5 ? lane : LOG2L == 6 ? lane / 2 : lane / 4);
     if (b >= ceil16(nb)) return 0u;
-    return LOG2L == 4 ? (uint32_t)__ldg((const unsigned short*)(cin + 32 + b))
-                      : (uint32_t)__ldg(cin + 32 + b);
+    return LOG2L == 4 ? (uint32_t)ld_dep((const unsigned short*)(cin + 32 + b))
+                      : (uint32_t)ld_dep(cin + 32 + b);
 }
 
 // Planes of 16 width bytes at byte b of a stream's width array: the sum of
@@ -382,16 +386,16 @@ __device__ __forceinline__ unsigned long long tile_unit_offset(const Item& it, u
     const unsigned t0 = min(t * NWARPS * BPU, wbytes);  // a multiple of 16
     unsigned pre = 0u, own = 0u;
 #pragma unroll 4
-    for (unsigned o = 16 * tid; o < t0; o += 16 * NTHREADS) pre += planes16(__ldg((const uint4*)(w + o)), nullptr, 0ull);
+    for (unsigned o = 16 * tid; o < t0; o += 16 * NTHREADS) pre += planes16(ld_dep((const uint4*)(w + o)), nullptr, 0ull);
     const unsigned u0 = (t * NWARPS + warp) * BPU;
     if (BPU == 8) {
         if (lane == 0 && u0 < wbytes) {
-            const uint2 v = __ldg((const uint2*)(w + u0));
+            const uint2 v = ld_dep((const uint2*)(w + u0));
             own = planes16(make_uint4(v.x, v.y, 0u, 0u), nullptr, 0ull);
         }
     } else {
         const unsigned o = u0 + 16 * lane;
-        if (lane < (int)(BPU / 16) && o < wbytes) own = planes16(__ldg((const uint4*)(w + o)), nullptr, 0ull);
+        if (lane < (int)(BPU / 16) && o < wbytes) own = planes16(ld_dep((const uint4*)(w + o)), nullptr, 0ull);
     }
     pre = __reduce_add_sync(FULL, pre);
     own = __reduce_add_sync(FULL, own);
@@ -407,7 +411,7 @@ __device__ __forceinline__ unsigned long long tile_unit_offset(const Item& it, u
         total += es.pre[v] + es.own[v];
     }
     constexpr unsigned long long PB = (1ull << LOG2L) / 8;
-    if (t + 1 == it.ntiles && tid == 0 && total * PB != __ldg((const unsigned long long*)it.cin + 3))
+    if (t + 1 == it.ntiles && tid == 0 && total * PB != ld_dep((const unsigned long long*)it.cin + 3))
         fail(ctl, ZC_ERR_FORMAT, item_idx);
     return off * PB;
 }
@@ -690,6 +694,22 @@ __device__ __forceinline__ int enc_raw(const Item& it, unsigned tile_in_item, Ti
     return 0;
 }
 
+// Copies n elements by the encoder warps of a CTA, eight loads in flight per
+// thread.  Not inlined: the batch kernel's coded tiles keep their registers.
+template <typename V>
+__device__ __noinline__ void copy_elems(V* dst, const V* src, unsigned long long n)
+{
+    unsigned long long i = threadIdx.x;
+    for (; i + 7 * NTHREADS < n; i += 8 * NTHREADS) {
+        V v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = ld_dep(src + i + k * NTHREADS);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) dst[i + k * NTHREADS] = v[k];
+    }
+    for (; i < n; i += NTHREADS) dst[i] = ld_dep(src + i);
+}
+
 template <int U>
 __device__ __forceinline__ void fin_raw(const Launch& P, const Item& it, unsigned item_idx,
                                         unsigned tile_in_item, unsigned g, const TileSlot& S)
@@ -709,14 +729,12 @@ __device__ __forceinline__ void fin_raw(const Launch& P, const Item& it, unsigne
         const uint8_t* src = (const uint8_t*)it.x + te0 * es;
         if (((uintptr_t)src & 15u) == 0) {
             const unsigned long long nv = bytes / 16;
-            for (unsigned long long i = tid; i < nv; i += NTHREADS)
-                ((uint4*)(out + base))[i] = __ldg((const uint4*)src + i);
+            copy_elems((uint4*)(out + base), (const uint4*)src, nv);
             for (unsigned long long i = nv * 16 + tid * 2; i < bytes; i += 2 * NTHREADS)
-                *(uint16_t*)(out + base + i) = __ldg((const unsigned short*)(src + i));
+                *(uint16_t*)(out + base + i) = ld_dep((const unsigned short*)(src + i));
         } else {
             // the input is only element-aligned: 2-byte copies
-            for (unsigned long long i = (unsigned long long)tid * 2; i < bytes; i += 2 * NTHREADS)
-                *(uint16_t*)(out + base + i) = __ldg((const unsigned short*)(src + i));
+            copy_elems((uint16_t*)(out + base), (const uint16_t*)src, bytes / 2);
         }
     } else if (tid == 0) {
         fail(P.ctl, ZC_ERR_CAPACITY, g);
@@ -1076,7 +1094,7 @@ __global__ void __launch_bounds__(NTHREADS) k_tile_map(const Item* items, unsign
     unsigned lo = 0, hi = n_items;
     while (hi - lo > 1) {
         const unsigned mid = (lo + hi) >> 1;
-        const unsigned b = by_chunk ? __ldg(&items[mid].chunk_begin) : __ldg(&items[mid].tile_begin);
+        const unsigned b = by_chunk ? ld_dep(&items[mid].chunk_begin) : ld_dep(&items[mid].tile_begin);
         if (b <= g) lo = mid;
         else hi = mid;
     }
@@ -1106,8 +1124,8 @@ __global__ void __launch_bounds__(GROUP_T) k_group_count(const Item* items, unsi
     int c = -1;
     unsigned t = 0;
     if (i < n_items) {
-        c = group_class(__ldg(&items[i].log2L));
-        t = __ldg(&items[i].ntiles);
+        c = group_class(ld_dep(&items[i].log2L));
+        t = ld_dep(&items[i].ntiles);
     }
 #pragma unroll
     for (int k = 0; k < GROUP_CLASSES; ++k) {
@@ -1277,7 +1295,7 @@ __global__ void __launch_bounds__(NTHREADS) k_wscan(const Launch P)
         if (k < ntile && b0 < wend) {
             const uint8_t* const w = it.cin + 32 + b0;
             if (bpt == 8) {
-                const uint2 v = __ldg((const uint2*)w);
+                const uint2 v = ld_dep((const uint2*)w);
                 sum = planes16(make_uint4(v.x, v.y, 0u, 0u), P.ctl, b0);
             } else {
                 const int nv = (int)min((unsigned long long)bpt, wend - b0) / 16;
@@ -1285,7 +1303,7 @@ __global__ void __launch_bounds__(NTHREADS) k_wscan(const Launch P)
                     uint4 v[4];
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
-                        v[q] = i + q < nv ? __ldg((const uint4*)w + i + q) : make_uint4(0u, 0u, 0u, 0u);
+                        v[q] = i + q < nv ? ld_dep((const uint4*)w + i + q) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
                     for (int q = 0; q < 4; ++q) sum += planes16(v[q], P.ctl, b0 + 16 * (i + q));
                 }
@@ -1309,7 +1327,7 @@ __global__ void __launch_bounds__(NTHREADS) k_wscan(const Launch P)
         const unsigned long long oslot = (unsigned long long)it.tile_begin * NWARPS + k;
         if (k < ntile && dcheck(P.ctl, oslot < P.ws_cap, oslot)) P.offs[oslot] = cex + wbase + ex;
         if (chunk + 1 == it.nchunks && tid == 0) {
-            const unsigned long long payload = __ldg((const unsigned long long*)it.cin + 3);
+            const unsigned long long payload = ld_dep((const unsigned long long*)it.cin + 3);
             if (cex + cagg != payload) fail(P.ctl, ZC_ERR_FORMAT, sm.item);
         }
     }
@@ -1330,13 +1348,19 @@ __device__ __forceinline__ void unit_raw_copy(const Item& it, int src_dtype, uns
 {
     const uint8_t* src = it.cin + 32;
     const int lane = threadIdx.x & 31;
-    for (int r = 0; r < DU; ++r) {
+    for (int r = 0; r < DU; r += 4) {  // four loads in flight
         const unsigned long long e = ue0 + (unsigned long long)r * 32 + lane;
-        if (e < it.n) {
-            const float v = src_dtype == ZC_F32 ? __ldg((const float*)src + e)
-                                                : bf16_to_f32(__ldg((const unsigned short*)src + e));
-            store_raw(it.raw_out, it.out_dtype, e, v);
+        float v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned long long ek = e + 32 * k;
+            v[k] = ek >= it.n ? 0.0f
+                   : src_dtype == ZC_F32 ? ld_dep((const float*)src + ek)
+                                         : bf16_to_f32(ld_dep((const unsigned short*)src + ek));
         }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (e + 32 * k < it.n) store_raw(it.raw_out, it.out_dtype, e + 32 * k, v[k]);
     }
 }
 
@@ -1464,10 +1488,10 @@ __device__ __forceinline__ unsigned long long local_unit_offset(const Item& it, 
     const unsigned v_pre = min(t * NWARPS * bpu / 16, v_end);
     unsigned pre = 0u;  // planes: at most 25 per block
 #pragma unroll 4
-    for (unsigned v = tid; v < v_pre; v += NTHREADS) pre += planes16(__ldg(w + v), nullptr, 0ull);
+    for (unsigned v = tid; v < v_pre; v += NTHREADS) pre += planes16(ld_dep(w + v), nullptr, 0ull);
     const unsigned v_lo = (t * NWARPS + warp) * (bpu / 16) + lane;
     unsigned own = 0u;
-    if (lane < (int)(bpu / 16) && v_lo < v_end) own = planes16(__ldg(w + v_lo), nullptr, 0ull);
+    if (lane < (int)(bpu / 16) && v_lo < v_end) own = planes16(ld_dep(w + v_lo), nullptr, 0ull);
     pre = __reduce_add_sync(FULL, pre);
     own = __reduce_add_sync(FULL, own);
     if (lane == 0) {
@@ -1481,7 +1505,7 @@ __device__ __forceinline__ unsigned long long local_unit_offset(const Item& it, 
         off += s_pre[v] + (v < warp ? s_own[v] : 0u);
         total += s_pre[v] + s_own[v];
     }
-    if (t + 1 == it.ntiles && tid == 0 && total * PB != __ldg((const unsigned long long*)it.cin + 3))
+    if (t + 1 == it.ntiles && tid == 0 && total * PB != ld_dep((const unsigned long long*)it.cin + 3))
         fail(ctl, ZC_ERR_FORMAT, item_idx);
     return off * PB;
 }
@@ -1525,7 +1549,7 @@ __device__ __forceinline__ void decompress_tile(const Launch& P)
     const unsigned slot = tile * NWARPS + warp;
     const unsigned bufs = (unsigned)__cvta_generic_to_shared(dsm) + warp * (2 * GBUF);
     float eb_in;
-    const int lg = check_header(it, P.ctl, idx, -1, eb_in, threadIdx.x == 0 && t == 0);
+    const int lg = check_header<!BATCH && !LOCAL>(it, P.ctl, idx, -1, eb_in, threadIdx.x == 0 && t == 0);
     long long loff = -1;  // the unit's payload offset, when this CTA finds it
     if (LOCAL && it.nchunks == 0 && lg >= 4)  // uniform in the CTA
         loff = (long long)local_unit_offset<DU>(it, lg, t, P.ctl, idx);

@@ -56,8 +56,8 @@ __device__ __forceinline__ void range_seg(Acc& a, const void* p, unsigned long l
     constexpr int VEC = 16 / sizeof(TX);
     constexpr int UNR = 4;
     auto one = [&](unsigned long long i) {
-        acc_one(a, sizeof(TX) == 4 ? __ldg((const float*)p + i)
-                                   : bf16_to_f32(__ldg((const unsigned short*)p + i)));
+        acc_one(a, sizeof(TX) == 4 ? ld_dep((const float*)p + i)
+                                   : bf16_to_f32(ld_dep((const unsigned short*)p + i)));
     };
     const unsigned long long skew = ((0ull - (unsigned long long)reinterpret_cast<uintptr_t>(p)) & 15ull) / sizeof(TX);
     const unsigned long long h = skew < n ? skew : n;
@@ -181,25 +181,25 @@ __device__ void range_finish(const RangeLaunch& P, Acc a)
 template <typename TX>
 __global__ void __launch_bounds__(256) k_range_one(const RangeLaunch P)
 {
-    grid_dep_wait();
+    const unsigned long long behind = grid_dep_wait_zero();
     grid_dep_launch();  // the compressor after it may be launched now (it waits for the bound)
     Acc a{FLT_MAX, -FLT_MAX, false};
     const unsigned long long gtid = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned long long gstride = (unsigned long long)gridDim.x * blockDim.x;
-    range_seg<TX>(a, P.one.x, P.one.n, gtid, gstride);
+    range_seg<TX>(a, (const uint8_t*)P.one.x + behind, P.one.n, gtid, gstride);
     range_finish(P, a);
 }
 
 template <typename TX>
 __global__ void __launch_bounds__(256) k_range_multi(const RangeLaunch P, const RangeSegs S)
 {
-    grid_dep_wait();
+    const unsigned long long behind = grid_dep_wait_zero();
     grid_dep_launch();  // the scatter pack after it may be launched now (it waits for the bound)
     Acc a{FLT_MAX, -FLT_MAX, false};
     const unsigned long long gtid = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned long long gstride = (unsigned long long)gridDim.x * blockDim.x;
     // last segment first, each from its end: the first segment's start is read last
-    for (unsigned k = P.n_segs; k-- > 0;) range_seg<TX>(a, S.ptr[k], S.cnt[k], gtid, gstride);
+    for (unsigned k = P.n_segs; k-- > 0;) range_seg<TX>(a, (const uint8_t*)S.ptr[k] + behind, S.cnt[k], gtid, gstride);
     range_finish(P, a);
 }
 

@@ -220,9 +220,17 @@ __device__ __forceinline__ void stage_in(const T* p, int nrem, bool vec, unsigne
         for (int k = 0; k < WPL; ++k) cp_async4_once(word_addr<T>(buf, k), src + k * 128);
     } else if (sizeof(T) == 2 && nrem > GELEMS && !first) {
         const unsigned* const src = (const unsigned*)((const uint8_t*)p - 2) + lane;
-#pragma unroll 4
-        for (int k = 0; k < WPL; ++k)
-            sts32(word_addr<T>(buf, k), __funnelshift_r(__ldcs(src + 32 * k), __ldcs(src + 32 * k + 1), 16));
+#pragma unroll 1
+        for (int k0 = 0; k0 < WPL; k0 += 4) {
+            uint32_t a[4], b[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                a[k] = ld_dep_once(src + 32 * (k0 + k));
+                b[k] = ld_dep_once(src + 32 * (k0 + k) + 1);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sts32(word_addr<T>(buf, k0 + k), __funnelshift_r(a[k], b[k], 16));
+        }
     } else if (sizeof(T) == 4) {
 #pragma unroll 8
         for (int k = 0; k < 32; ++k) {
@@ -230,10 +238,14 @@ __device__ __forceinline__ void stage_in(const T* p, int nrem, bool vec, unsigne
             cp_async_ca<4>(elem_addr<T>(buf, e), p + min(e, nrem - 1));
         }
     } else {
-#pragma unroll 8
-        for (int k = 0; k < 32; ++k) {
-            const int e = k * 32 + lane;
-            sts16(elem_addr<T>(buf, e), __ldg((const unsigned short*)p + min(e, nrem - 1)));
+#pragma unroll 1
+        for (int k0 = 0; k0 < 32; k0 += 8) {
+            uint32_t v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                v[k] = ld_dep((const unsigned short*)p + min((k0 + k) * 32 + lane, nrem - 1));
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sts16(elem_addr<T>(buf, (k0 + k) * 32 + lane), v[k]);
         }
     }
     cp_commit();
@@ -716,12 +728,12 @@ struct PlaneSrc {
     __device__ __forceinline__ uint32_t u32(int off) const
     {
         if (SMEM) return lds32(sp + off);
-        return __ldg((const unsigned*)(gp + off));
+        return ld_dep((const unsigned*)(gp + off));
     }
     __device__ __forceinline__ uint32_t u16(int off) const
     {
         if (SMEM) return lds16(sp + off);
-        return __ldg((const unsigned short*)(gp + off));
+        return ld_dep((const unsigned short*)(gp + off));
     }
 };
 

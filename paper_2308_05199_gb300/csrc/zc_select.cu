@@ -61,23 +61,23 @@ __device__ __forceinline__ void load_span4(const Item& it, bool vec, unsigned lo
     if (it.x_dtype == ZC_F32) {
         const float* p = (const float*)it.x + s0 + i0;
         if (vec && i0 + 4 <= cnt) {
-            const float4 w = __ldg((const float4*)p);
+            const float4 w = ld_dep((const float4*)p);
             v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w;
         } else {
 #pragma unroll
-            for (int m = 0; m < 4; ++m) v[m] = i0 + m < cnt ? __ldg(p + m) : 0.0f;
+            for (int m = 0; m < 4; ++m) v[m] = i0 + m < cnt ? ld_dep(p + m) : 0.0f;
         }
     } else {
         const unsigned short* p = (const unsigned short*)it.x + s0 + i0;
         if (vec && i0 + 4 <= cnt) {
-            const uint2 w = __ldg((const uint2*)p);
+            const uint2 w = ld_dep((const uint2*)p);
             v[0] = __uint_as_float(w.x << 16);
             v[1] = __uint_as_float(w.x & 0xffff0000u);
             v[2] = __uint_as_float(w.y << 16);
             v[3] = __uint_as_float(w.y & 0xffff0000u);
         } else {
 #pragma unroll
-            for (int m = 0; m < 4; ++m) v[m] = i0 + m < cnt ? bf16_to_f32(__ldg(p + m)) : 0.0f;
+            for (int m = 0; m < 4; ++m) v[m] = i0 + m < cnt ? bf16_to_f32(ld_dep(p + m)) : 0.0f;
         }
     }
 }
