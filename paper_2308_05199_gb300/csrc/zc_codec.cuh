@@ -271,10 +271,11 @@ __device__ __forceinline__ int planes16(const uint4& v, Ctl* ctl, unsigned long 
 // 2-byte units is shifted on the way out), all of them in flight at once, and
 // 16-byte stores take them out.  (Copied through registers, four 4-byte loads
 // at a time, a 4 KiB segment took eight round trips to L2.)  The staged bytes
-// are dead afterwards: their L2 lines (the segment owns whole 128-byte lines)
-// are dropped without a write-back, so the ring costs no DRAM traffic as long
+// are dead afterwards: the L2 lines of 128 bytes that lie wholly in the segment
+// (of SEG bytes; all of them when the workspace starts on such a line, as it need
+// not) are dropped without a write-back, so the ring costs no DRAM traffic as long
 // as a tile's lines stay in L2 until it is stored.
-template <int UNIT>
+template <int UNIT, int SEG>
 __device__ __forceinline__ void ring_copy(uint8_t* dst, const uint8_t* src, int len, unsigned buf)
 {
     constexpr int W = UNIT == 2 ? 4 : UNIT;  // bytes per asynchronous copy
@@ -314,9 +315,9 @@ __device__ __forceinline__ void ring_copy(uint8_t* dst, const uint8_t* src, int 
         }
         __syncwarp();  // the buffer is free
     }
-    for (int l = lane; l < (len + 127) >> 7; l += 32)
-        asm volatile("discard.global.L2 [%0], 128;" ::"l"(__cvta_generic_to_global(src + 128 * l))
-                     : "memory");
+    const int skew = (int)(0u - (unsigned)(uintptr_t)src) & 127;  // to the first whole line
+    for (int l = skew + 128 * lane; l < len && l + 128 <= SEG; l += 128 * 32)
+        asm volatile("discard.global.L2 [%0], 128;" ::"l"(__cvta_generic_to_global(src + l)) : "memory");
 }
 
 // Packed mode (one chain through many streams): the first tile of a stream
@@ -622,7 +623,7 @@ __device__ __forceinline__ void fin_tile(const Launch& P, const Item& it, unsign
     const unsigned long long end = base + payload;  // unpadded end of this tile's payload
     if (base + payload <= cap) {
         if (dcheck(P.ctl, S.segsz[warp] <= seg_bytes(U), g))
-            ring_copy<PB>(out + base + segoff, seg, S.segsz[warp], buf);
+            ring_copy<PB, seg_bytes(U)>(out + base + segoff, seg, S.segsz[warp], buf);
     } else if (tid == 0) {
         fail(P.ctl, ZC_ERR_CAPACITY, g);
     }
