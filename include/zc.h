@@ -423,7 +423,8 @@ int zc_mlp_sgd(float* d_params, float* d_vel, const float* d_grad, float lr, flo
  * each minibatch the gradient, then the update, as zc_mlp_grad and zc_mlp_sgd
  * define them, sums in a fixed order.  d_grad receives the last minibatch's
  * gradient, d_losses[ceil(N / batch)] every minibatch's loss.  Scratch as for
- * zc_mlp_grad of `batch` rows (large minibatches use it). */
+ * zc_mlp_grad of min(batch, N) rows, always (minibatches above 1024 rows use
+ * it, and GPUs without room for a cluster of 16 CTAs). */
 int zc_mlp_fit_epoch(float* d_params, float* d_vel, float* d_grad, const float* d_norm,
                      const float* d_x, const float* d_t, const int* d_idx, int N, int batch,
                      double lr, double momentum, float* d_losses, void* d_scratch,

@@ -1121,6 +1121,10 @@ int zc_mlp_fit_epoch(float* d_params, float* d_vel, float* d_grad, const float* 
         d_x == nullptr || d_t == nullptr || d_idx == nullptr || d_losses == nullptr)
         return ZC_ERR_ARG;
     if (batch > N) batch = N;
+    // (whichever way the epoch runs: what is valid does not depend on the device)
+    if (d_scratch == nullptr || scratch_bytes < zc_mlp_scratch_bytes(batch) ||
+        (reinterpret_cast<uintptr_t>(d_scratch) & 3) != 0)
+        return ZC_ERR_ARG;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(FC);
     cfg.blockDim = dim3(FM);
