@@ -456,13 +456,17 @@ __device__ __forceinline__ void expand_bf16(unsigned buf)
 
 // The general path of a group: any width, any rounding, errors.  `bad`: rows
 // that hold a value whose fast rounding is not proven (near a tie, or beyond
-// 2^20: `far`).  Bad rows are requantized exactly, a lane per element, and
-// their values replaced by q 2eb, whose fast rounding is q again (|q| < 2^20,
-// heads apart 2^21: x' and inv are off by at most 2^-24 relatively, so x' inv is
-// within 1/4 of q); with `far` set every row is requantized and the buffer then holds the
-// rounding results themselves.  Then 32-bit deltas, byte by byte.  Not
+// 2^20: `far`).  Bad rows are settled a lane per element: q next to x inv is at
+// most one off, and the residual e = x - q 2eb decides (exact where |e| is near
+// eb: there it is a multiple of ulp(eb), see quantize).  Their values are replaced
+// by q 2eb, whose fast rounding is q again (|q| < 2^20, heads apart 2^21: x' and inv
+// are off by at most 2^-24 relatively, so x' inv is within 1/4 of q).  With `far`
+// set every row is quantized by quantize(), errors and all, and the buffer then holds
+// the rounding results themselves.  Then 32-bit deltas, byte by byte.  Not
 // inlined: a few groups in a hundred come here (near-tie values, |q| >=
-// 16000), and the fast path keeps its registers.
+// 16000), and the fast path keeps its registers.  Where every row is bad (bytes at
+// 2eb = 2: each odd one is a tie; 2^24 of them, L = 32) compression takes 42 us,
+// where quantize() for bad rows too took 61.
 template <int LOG2L, bool HEADS, bool BF>
 __device__ __noinline__ int encode_rows_general(const EncArgs A, unsigned bad, bool far, int* err)
 {
@@ -471,16 +475,27 @@ __device__ __noinline__ int encode_rows_general(const EncArgs A, unsigned bad, b
     if (BF) expand_bf16(A.buf);
     // q 2eb of a value near FLT_MAX may overflow (x = FLT_MAX, 2eb = 1.5 2^126: q =
     // 3); |q| < 2^21 keeps it finite for a 2eb below 2^107
-    if (A.two_eb >= 0x1p107f) far = true;
-    unsigned todo = far ? FULL : bad;
-    while (todo) {  // warp-uniform
-        const int r = __ffs(todo) - 1;
-        todo &= todo - 1;
-        const unsigned p = elem_addr<float>(A.buf, r * 32 + lane);
-        const float x = __uint_as_float(lds32(p));
-        int q;
-        *err |= quantize(x, A.eb, A.two_eb, A.inv, q);
-        sts32(p, far ? (uint32_t)(q + QBIAS) : __float_as_uint(__fmul_rn(__int2float_rn(q), A.two_eb)));
+    if (bad != 0u && A.two_eb >= 0x1p107f) far = true;
+    if (far) {
+#pragma unroll 1
+        for (int r = 0; r < GROWS; ++r) {
+            const unsigned p = elem_addr<float>(A.buf, r * 32 + lane);
+            int q;
+            *err |= quantize(__uint_as_float(lds32(p)), A.eb, A.two_eb, A.inv, q);
+            sts32(p, (uint32_t)(q + QBIAS));
+        }
+    } else {
+        while (bad) {  // warp-uniform
+            const unsigned p = elem_addr<float>(A.buf, (__ffs(bad) - 1) * 32 + lane);
+            bad &= bad - 1;
+            const float x = __uint_as_float(lds32(p));
+            const float t = __fmaf_rn(x, A.inv, 12582912.0f);
+            float q = __fsub_rn(t, 12582912.0f);
+            const int e = __float_as_int(__fmaf_rn(-q, A.two_eb, x));
+            // |e| > eb, or = eb at an odd q (positive floats order like their bits)
+            if ((e & 0x7fffffff) + (__float_as_int(t) & 1) > __float_as_int(A.eb)) q += e < 0 ? -1.0f : 1.0f;
+            sts32(p, __float_as_uint(__fmul_rn(q, A.two_eb)));
+        }
     }
     __syncwarp();
     int d[32];
