@@ -375,7 +375,8 @@ struct EncShared {
 // Payload offset of this warp's unit of a received stream without a width
 // scan: the encoder warps of the CTA sum the width bytes before the tile and
 // of its units (16 bytes per thread and load).  The item's last tile checks
-// the total against the header's payload size, as the scan does.
+// the total against the header's payload size, as the scan does, and every tile
+// reports its own bytes that no width can have, padding included.
 template <int LOG2L, int U>
 __device__ __forceinline__ unsigned long long tile_unit_offset(const Item& it, unsigned t, Ctl* ctl,
                                                                unsigned item_idx, EncShared& es)
@@ -392,11 +393,11 @@ __device__ __forceinline__ unsigned long long tile_unit_offset(const Item& it, u
     if (BPU == 8) {
         if (lane == 0 && u0 < wbytes) {
             const uint2 v = ld_dep((const uint2*)(w + u0));
-            own = planes16(make_uint4(v.x, v.y, 0u, 0u), nullptr, 0ull);
+            own = planes16(make_uint4(v.x, v.y, 0u, 0u), ctl, u0);
         }
     } else {
         const unsigned o = u0 + 16 * lane;
-        if (lane < (int)(BPU / 16) && o < wbytes) own = planes16(ld_dep((const uint4*)(w + o)), nullptr, 0ull);
+        if (lane < (int)(BPU / 16) && o < wbytes) own = planes16(ld_dep((const uint4*)(w + o)), ctl, o);
     }
     pre = __reduce_add_sync(FULL, pre);
     own = __reduce_add_sync(FULL, own);
@@ -1484,7 +1485,8 @@ __device__ __forceinline__ void unit_decode(const Launch& P, const Item& it, uns
 // t sums the plane bytes of the item's blocks before its tile itself and its
 // warps' units (one value per warp), which gives every warp its unit's payload
 // offset; the item's last tile checks the total against the header's payload
-// size, as the width scan does.  Called by every thread of the CTA (coded
+// size, as the width scan does, and every tile reports its own bytes that no
+// width can have, padding included.  Called by every thread of the CTA (coded
 // streams only: lg >= 4).
 template <int DU>
 __device__ __forceinline__ unsigned long long local_unit_offset(const Item& it, int lg, unsigned t,
@@ -1506,7 +1508,7 @@ __device__ __forceinline__ unsigned long long local_unit_offset(const Item& it, 
     for (unsigned v = tid; v < v_pre; v += NTHREADS) pre += planes16(ld_dep(w + v), nullptr, 0ull);
     const unsigned v_lo = (t * NWARPS + warp) * (bpu / 16) + lane;
     unsigned own = 0u;
-    if (lane < (int)(bpu / 16) && v_lo < v_end) own = planes16(ld_dep(w + v_lo), nullptr, 0ull);
+    if (lane < (int)(bpu / 16) && v_lo < v_end) own = planes16(ld_dep(w + v_lo), ctl, 16ull * v_lo);
     pre = __reduce_add_sync(FULL, pre);
     own = __reduce_add_sync(FULL, own);
     if (lane == 0) {
