@@ -780,7 +780,7 @@ __device__ __forceinline__ int rows_before(int tot)
     return s - tot;
 }
 
-// Four consecutive values x^ = q 2eb from the bits of q + 1.5 2^23.
+// Four consecutive values x^ = q 2eb from the bits of q + 1.5 2^23 (|q| <= 2^22).
 template <typename Emit>
 __device__ __forceinline__ void emit_bits(int c, const int b[4], f32x2 te2, const Emit& emit)
 {
@@ -788,6 +788,17 @@ __device__ __forceinline__ void emit_bits(int c, const int b[4], f32x2 te2, cons
     float v[4];
     up2(mul2(add2(pk2(__int_as_float(b[0]), __int_as_float(b[1])), nmag), te2), v[0], v[1]);
     up2(mul2(add2(pk2(__int_as_float(b[2]), __int_as_float(b[3])), nmag), te2), v[2], v[3]);
+    emit(c, v);
+}
+
+// The same from any q: a stream's heads and wide deltas can sum to levels beyond
+// 2^22, which no encoder writes but which have a value all the same.
+template <typename Emit>
+__device__ __forceinline__ void emit_ints(int c, const int q[4], f32x2 te2, const Emit& emit)
+{
+    float v[4];
+    up2(mul2(pk2(__int2float_rn(q[0]), __int2float_rn(q[1])), te2), v[0], v[1]);
+    up2(mul2(pk2(__int2float_rn(q[2]), __int2float_rn(q[3])), te2), v[2], v[3]);
     emit(c, v);
 }
 
@@ -821,15 +832,15 @@ __device__ __forceinline__ void decode_rows_wide(const PlaneSrc<SMEM>& P, int np
         for (int i = 0; i < 32; ++i) tot += delta(i);
     }
     // (a head reaches its block's later rows through the sums)
-    int q = QBIAS + (HEADS ? h0 : 0) + (L >= 64 ? rows_before<RPB>(tot + (HEADS ? h0 : 0)) : 0);
+    int q = (HEADS ? h0 : 0) + (L >= 64 ? rows_before<RPB>(tot + (HEADS ? h0 : 0)) : 0);
     const f32x2 te2 = pk2(two_eb, two_eb);
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-        if (L == 16 && c == 4) q = QBIAS + (HEADS ? h16 : 0);
+        if (L == 16 && c == 4) q = HEADS ? h16 : 0;
         int b[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) b[i] = q += delta(4 * c + i);
-        emit_bits(c, b, te2, emit);
+        emit_ints(c, b, te2, emit);
     }
 }
 
@@ -906,17 +917,17 @@ __device__ __forceinline__ void decode_rows(const PlaneSrc<SMEM>& P, int np, int
                 for (int k = 0; k < 8; ++k) t = __dp4a(w[k], 0x01010101u, t);
                 tot = (int)t - 32 * 128;
             }
-            int q = QBIAS + h0 + (L >= 64 ? rows_before<RPB>(tot + h0) : 0);
+            int q = h0 + (L >= 64 ? rows_before<RPB>(tot + h0) : 0);
 #pragma unroll
             for (int cc = 0; cc < 8; ++cc) {
-                if (L == 16 && cc == 4) q = QBIAS + h16;
+                if (L == 16 && cc == 4) q = h16;
                 int b[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int e = 4 * cc + i;
                     b[i] = q += (int)__byte_perm(w[e & 7], 0u, 0x4440 + (e >> 3)) - 128;
                 }
-                emit_bits(cc, b, te2, emit);
+                emit_ints(cc, b, te2, emit);
             }
             return;
         }
@@ -936,7 +947,8 @@ __device__ __forceinline__ void decode_rows(const PlaneSrc<SMEM>& P, int np, int
         a[k] = __byte_perm(w[k], h[k], 0x6240);
         a[k + 8] = __byte_perm(w[k], h[k], 0x7351);
     }
-    int q = QBIAS + (HEADS ? h0 : 0);
+    // (without heads |q| <= 128 (2^15 - 1) < 2^22)
+    int q = HEADS ? h0 : QBIAS;
     if (L >= 64) {
         int tot = HEADS ? h0 : 0;
 #pragma unroll
@@ -945,12 +957,13 @@ __device__ __forceinline__ void decode_rows(const PlaneSrc<SMEM>& P, int np, int
     }
 #pragma unroll
     for (int cc = 0; cc < 8; ++cc) {
-        if (L == 16 && cc == 4) q = QBIAS + (HEADS ? h16 : 0);
+        if (L == 16 && cc == 4) q = HEADS ? h16 : QBIAS;
         int b[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)  // one element of the pair added per dot product
             b[i] = q = __dp2a_lo((int)a[(4 * cc + i) & 15], cc < 4 ? 0x0001 : 0x0100, q);
-        emit_bits(cc, b, te2, emit);
+        if (HEADS) emit_ints(cc, b, te2, emit);
+        else emit_bits(cc, b, te2, emit);
     }
 }
 
