@@ -168,7 +168,7 @@ def kernel_times(samples):
 # The sources the encoder kernels (k_compress, k_batch, k_reduce, k_scatter) are
 # built from: a DRAM-traffic figure taken with ncu stays valid while these are
 # unchanged.
-ENCODER_SOURCES = ("zc_device.cuh", "zc_codec.cuh", "zc_launch.h", "zc_kbatch.cu",
+ENCODER_SOURCES = ("zc_device.cuh", "zc_rows.cuh", "zc_codec.cuh", "zc_launch.h", "zc_kbatch.cu",
                    "zc_kenc.cu")
 
 
