@@ -99,8 +99,9 @@ size_t zc_raw_stream_bytes(uint64_t n, int dtype);
  * `n_items` items (1 for single calls, P for batched ring steps and scatter
  * packs, M for batched compression).  Host-side arithmetic only.  Besides the
  * look-back records it holds the encoder CTAs' tile rings (staged payload of
- * the tiles in flight, at most 200 KB per CTA, up to 608 CTAs: at most
- * 124.5 MB); a smaller workspace still works, with fewer encoder CTAs. */
+ * the tiles in flight, at most 200 KB per CTA, up to 608 of them: at most
+ * 124.5 MB; 456 CTAs run at a time on 152 SMs); a smaller workspace still works,
+ * with fewer encoder CTAs.  A workspace is 16-byte aligned. */
 size_t zc_workspace_bytes(uint64_t n_total, int n_items);
 
 /* Zero the workspace (cudaMemsetAsync) and stamp it as initialised.  Call
@@ -272,7 +273,7 @@ size_t zc_batch_max_bytes(int n_msgs, const zc_message* h_msgs);
 /* Plan the compression of h_msgs[0 .. n_msgs) into d_packed (16-byte
  * aligned).  tile_chunks: 4, 8, 16, or 0 for the current default
  * (zc_set_tile_chunks); grid: CTAs to launch (at most one per tile, per
- * ring of the workspace and 4 per SM), 0 = as many as allowed.  Validates
+ * ring of the workspace and 3 per SM), 0 = as many as allowed.  Validates
  * every message (ZC_ERR_ARG), checks that packed_cap holds at least every
  * header and width array (ZC_ERR_CAPACITY; the payload is checked on the
  * device), and copies the table to d_table with a synchronous cudaMemcpy. */
@@ -329,7 +330,8 @@ int zc_batch_set_grouped(zc_batch* plan, int grouped);
 
 /* Autotuner for batched compression.  Times zc_compress_batch on the given
  * messages for every candidate tile size (4, 8, 16 chunks) and grid (1, 2 and
- * 4 CTAs per SM, and as many as allowed), and, with tune_block != 0, every
+ * 4 CTAs per SM, and as many as allowed; more than 3 per SM are cut to 3, so the
+ * last two run alike), and, with tune_block != 0, every
  * block size (16 .. 128, applied to all non-raw messages).  Each candidate
  * runs once untimed and `reps` times timed with CUDA events on s; its score
  * is the median time plus, for link_gbs > 0, the time to send the packed

@@ -68,7 +68,9 @@ int qparams(double eb_abs, float* eb, float* two, float* inv)
 // tile-to-item map of multi-item encoder launches (u32 entries); then the
 // encoder CTAs' tile rings: ring_ctas(cap) rings of the largest tile size.
 constexpr uint64_t WS_ARRAYS = 9;
-constexpr uint64_t RING_CTAS_MAX = 152 * 4;  // rings of the largest workspace
+// Rings of the largest workspace: four per SM of 152, while ENC_CTAS_PER_SM CTAs are
+// resident; the size that callers have asked for and allocated stays what it was.
+constexpr uint64_t RING_CTAS_MAX = 152 * 4;
 constexpr uint64_t RING_UNIT = ring_cta_bytes(unit_rows(16));  // the largest ring of any tile size
 static_assert(RING_UNIT >= ring_cta_bytes(unit_rows(8)) && RING_UNIT >= ring_cta_bytes(unit_rows(4)), "ring unit");
 

@@ -89,13 +89,17 @@ __device__ __forceinline__ unsigned long long ceil16(unsigned long long v)
 // runs; grid_dep_wait() blocks until that kernel has completed and its memory
 // operations are visible (it returns at once in a kernel launched without
 // the attribute).  grid_dep_launch() lets the dependent kernel start early.
-// The codec's kernels (but the range pass) are launched this way and call both
-// first thing, in this order: the launch of a kernel, and its CTAs' way onto the
+// The codec's kernels but large range passes, most tile maps and the training
+// kernels are launched this way: the launch of a kernel, and its CTAs' way onto the
 // SMs, overlap the end of the one before (a 4 MiB signal, there and back: 23.1 ->
-// 19.9 us; five-rank recursive doubling of 1M elements: 118 -> 113).  A kernel that lets the next one
-// start only after its own wait keeps every kernel before it complete, so
-// what the next one reads ahead of its own wait (the decoder its stream's
-// header, the tile map its items) is not still being written.
+// 19.9 us; five-rank recursive doubling of 1M elements: 118 -> 113).  What keeps
+// this safe: every such kernel waits before it completes, so a kernel whose wait is
+// over finds everything before it complete; and all but two wait first, then let
+// the next one start.  Those two are only ever launched right behind a width
+// scan, which has waited itself: the tile map of a fused step (it reads its item
+// table ahead of its wait) and the decoder of a scanned stream (its header).  Neither
+// that table nor that stream is still being written then, and what comes after them
+// waits as always.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

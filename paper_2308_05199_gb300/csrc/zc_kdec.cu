@@ -45,7 +45,7 @@ static cudaError_t decompress_u(const Launch& P, unsigned grid, cudaStream_t s, 
     const cudaError_t e = smem_limit<k_decompress<false, false, DU>>(DEC_SMEM_BYTES);
     if (e != cudaSuccess) return e;
     // launched dependent on the width scan just before it on the stream: its
-    // CTAs read their headers and width bytes while the scan still runs
+    // CTAs read their headers while the scan still runs
     return launch_after(k_decompress<false, false, DU>, grid, NTHREADS, DEC_SMEM_BYTES, s, P);
 }
 

@@ -24,9 +24,11 @@ inline cudaError_t smem_limit(int bytes)
     return e;
 }
 
-// Launches a kernel that begins with grid_dep_wait() dependent on the kernel
-// just before it on the stream (programmatic serialisation; nothing changes
-// where the work before it is not a kernel).
+// Launches a kernel dependent on the kernel just before it on the stream
+// (programmatic serialisation; nothing changes where the work before it is not a
+// kernel).  The kernel calls grid_dep_wait() before it touches what earlier work
+// on the stream wrote or still reads (the rule, and its two exceptions, stand at
+// grid_dep_wait()).
 template <typename... A>
 inline cudaError_t launch_after(void (*k)(A...), unsigned grid, unsigned threads, int smem, cudaStream_t s,
                                 const A&... args)

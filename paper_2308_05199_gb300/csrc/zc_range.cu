@@ -44,7 +44,7 @@ __device__ __forceinline__ void acc_vec(Acc& a, const uint4 v)
 // before the first 16-byte boundary and behind the last one.  (A segment off
 // that boundary was read by single elements throughout: the range pass took
 // 121 of the 194 us of a 200 MB scatter pack of 8 such segments; the whole
-// call takes 102 now.)
+// call takes 101 now.)
 // Measured on 512 MiB: 6.1 TB/s with streaming loads at 3 to 6 CTAs per SM,
 // 5.3-5.4 TB/s with __ldg or ld.global.cg.  The pass runs from the end of
 // the segment to its start, so the last lines it reads are the first ones
@@ -241,7 +241,7 @@ __global__ void k_ws_init(Ctl* c)
     c->magic = WS_MAGIC;
 }
 
-constexpr unsigned RANGE_SMALL_GRID = 152;  // at most a CTA per SM (1.2M elements)
+constexpr unsigned RANGE_SMALL_GRID = 152;  // the SMs of a whole GPU: a CTA each at most (1.2M elements)
 
 cudaError_t launch_range(const RangeLaunch& R, unsigned grid, cudaStream_t s)
 {
