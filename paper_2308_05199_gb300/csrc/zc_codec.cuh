@@ -228,6 +228,13 @@ __device__ __forceinline__ uint32_t load_widths(const uint8_t* cin, unsigned lon
                       : (uint32_t)ld_dep(cin + 32 + b);
 }
 
+// Whether 16 bytes can all be widths.
+__device__ __forceinline__ bool widths_fit(const uint4& v)
+{
+    const unsigned up = 0x01010101u * (127 - ZC_MAX_WIDTH);  // bit 7 of a byte: above the largest
+    return ((v.x | (v.x + up) | v.y | (v.y + up) | v.z | (v.z + up) | v.w | (v.w + up)) & 0x80808080u) == 0u;
+}
+
 // Planes of 16 width bytes at byte b of a stream's width array: the sum of
 // w + 1 over the nonzero widths, four bytes at a time (a width above the
 // format's counts as none and is reported when `ctl` is set).
@@ -375,8 +382,8 @@ struct EncShared {
 // Payload offset of this warp's unit of a received stream without a width
 // scan: the encoder warps of the CTA sum the width bytes before the tile and
 // of its units (16 bytes per thread and load).  The item's last tile checks
-// the total against the header's payload size, as the scan does, and every tile
-// reports its own bytes that no width can have, padding included.
+// the total against the header's payload size, as the scan does, and the last
+// width bytes, whose padding may lie beyond the last group of rows (blocks of 128).
 template <int LOG2L, int U>
 __device__ __forceinline__ unsigned long long tile_unit_offset(const Item& it, unsigned t, Ctl* ctl,
                                                                unsigned item_idx, EncShared& es)
@@ -393,11 +400,11 @@ __device__ __forceinline__ unsigned long long tile_unit_offset(const Item& it, u
     if (BPU == 8) {
         if (lane == 0 && u0 < wbytes) {
             const uint2 v = ld_dep((const uint2*)(w + u0));
-            own = planes16(make_uint4(v.x, v.y, 0u, 0u), ctl, u0);
+            own = planes16(make_uint4(v.x, v.y, 0u, 0u), nullptr, 0ull);
         }
     } else {
         const unsigned o = u0 + 16 * lane;
-        if (lane < (int)(BPU / 16) && o < wbytes) own = planes16(ld_dep((const uint4*)(w + o)), ctl, o);
+        if (lane < (int)(BPU / 16) && o < wbytes) own = planes16(ld_dep((const uint4*)(w + o)), nullptr, 0ull);
     }
     pre = __reduce_add_sync(FULL, pre);
     own = __reduce_add_sync(FULL, own);
@@ -413,7 +420,9 @@ __device__ __forceinline__ unsigned long long tile_unit_offset(const Item& it, u
         total += es.pre[v] + es.own[v];
     }
     constexpr unsigned long long PB = (1ull << LOG2L) / 8;
-    if (t + 1 == it.ntiles && tid == 0 && total * PB != ld_dep((const unsigned long long*)it.cin + 3))
+    if (t + 1 == it.ntiles && tid == 0 &&
+        (total * PB != ld_dep((const unsigned long long*)it.cin + 3) ||
+         (LOG2L == 7 && wbytes != 0u && !widths_fit(ld_dep((const uint4*)(w + wbytes - 16))))))
         fail(ctl, ZC_ERR_FORMAT, item_idx);
     return off * PB;
 }
