@@ -1497,7 +1497,7 @@ __device__ __forceinline__ void unit_decode(const Launch& P, const Item& it, uns
 // size, as the width scan does, and every tile reports its own bytes that no
 // width can have, padding included.  Called by every thread of the CTA (coded
 // streams only: lg >= 4).
-template <int DU>
+template <bool BATCH, int DU>
 __device__ __forceinline__ unsigned long long local_unit_offset(const Item& it, int lg, unsigned t,
                                                                 Ctl* ctl, unsigned item_idx)
 {
@@ -1531,8 +1531,18 @@ __device__ __forceinline__ unsigned long long local_unit_offset(const Item& it, 
         off += s_pre[v] + (v < warp ? s_own[v] : 0u);
         total += s_pre[v] + s_own[v];
     }
-    if (t + 1 == it.ntiles && tid == 0 && total * PB != ld_dep((const unsigned long long*)it.cin + 3))
-        fail(ctl, ZC_ERR_FORMAT, item_idx);
+    if (t + 1 == it.ntiles && tid == 0) {
+        const unsigned long long payload = ld_dep((const unsigned long long*)it.cin + 3);
+        if (total * PB != payload) {
+            // a batch's small items may have widths in their padding, as long as
+            // what these stand for lies inside the stream's room
+            unsigned pad = 0u;
+            if (BATCH && it.ntiles <= DEC_LOCAL_TILES &&
+                32ull + ceil16(nb) + (lg >= 8 ? ceil16(3ull * nb) : 0ull) + total * PB <= it.cin_cap)
+                for (unsigned long long b = nb; b < ceil16(nb); ++b) pad += planes_of(ld_dep(it.cin + 32 + b));
+            if ((total - pad) * PB != payload) fail(ctl, ZC_ERR_FORMAT, item_idx);
+        }
+    }
     return off * PB;
 }
 
@@ -1578,7 +1588,7 @@ __device__ __forceinline__ void decompress_tile(const Launch& P)
     const int lg = check_header<!BATCH && !LOCAL>(it, P.ctl, idx, -1, eb_in, threadIdx.x == 0 && t == 0);
     long long loff = -1;  // the unit's payload offset, when this CTA finds it
     if (LOCAL && it.nchunks == 0 && lg >= 4)  // uniform in the CTA
-        loff = (long long)local_unit_offset<DU>(it, lg, t, P.ctl, idx);
+        loff = (long long)local_unit_offset<BATCH, DU>(it, lg, t, P.ctl, idx);
     // the width scan's offsets are read from here on: a single-stream decoder
     // launched dependent on the scan has looked up its tile and checked the
     // header while the scan ran, and waits for it now.  Every thread passes

@@ -51,3 +51,26 @@ def test_padding_bytes(zc, block, n, value):
         d = zc.BatchDecompress(s, off, [torch.zeros(n, device="cuda")])
         d.run()
         assert d.ws.status()[0] == zc.ERR_FORMAT, at
+
+
+@pytest.mark.parametrize("n", [9, 500, 17 * 1024, 4 * 16384 - 700])
+@pytest.mark.parametrize("block", [16, 32, 64, 128])
+def test_small_items_of_a_batch(zc, block, n):
+    """Widths in the padding of a batch's small items are let through where the planes
+    they stand for would lie inside the item's room, and change no value."""
+    made = stream(n, block, 0, 2)
+    if made is None:
+        pytest.skip("no padding at this size")
+    x, s = made
+    room = torch.zeros(s.numel() + 1024, dtype=torch.uint8, device="cuda")
+    room[:s.numel()] = s
+    off = torch.tensor([0, room.numel()], dtype=torch.int64, device="cuda")
+    y = torch.zeros(n, device="cuda")
+    d = zc.BatchDecompress(room, off, [y])
+    d.run()
+    assert d.ws.status()[0] == 0
+    good = oracle.decompress(oracle.compress(x, EB, block.bit_length() - 1), n)
+    np.testing.assert_array_equal(y.cpu().numpy(), good)
+    ws = zc.Workspace(n)
+    zc.decompress(room, n, ws=ws)
+    assert ws.status()[0] == zc.ERR_FORMAT
